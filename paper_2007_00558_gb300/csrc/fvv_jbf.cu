@@ -14,11 +14,11 @@
 // are valid codes; the background signal is neither a source nor filled.
 // One pass, out of place.
 //
-// The filter reads 2 + 3 bytes and writes 2 bytes per pixel: it is bound by
-// HBM bandwidth once the few pixels without depth, the only ones that visit
-// their window, no longer hold up whole warps (see k_jbf).
+// The filter reads 2 + 3 bytes and writes 2 bytes per pixel, but is bound by
+// instruction issue in the windows of the pixels without depth (see k_jbf).
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 
 #include "fvv_jbf.h"
 #include "fvv_runtime.h"
@@ -33,37 +33,52 @@ __device__ __forceinline__ float code_to_float(uint32_t d)   // exact for d < 2^
 }
 
 // A CTA filters a kTileW x kTileH tile of camera blockIdx.z.  Phase 1
-// stages the tile and its halo (codes and colour bytes) in shared memory:
-// the tile's own columns as 16-byte loads and stores when the rows are
-// 16-byte aligned, the halo columns and ragged edges element by element.
-// Phase 2 writes the tile's codes back out 8 at a time and lists the pixels
-// without one.  Phase 3 deals the listed pixels out to the threads, so a
-// tile's few holes are filtered by many threads at once instead of idling
-// the rest of their warps; each filtered pixel walks its window in shared
-// memory in the stated order (the radius is a template parameter, so the
-// window unrolls and its loads are in flight together) and overwrites its
-// output.
-constexpr int kTileW = 64, kTileH = 16, kThreads = 256;
+// stages the tile and its halo (codes and colour bytes) in shared memory: 16
+// bytes a lane when the rows are 16-byte aligned, else element by element,
+// neighbouring lanes on neighbouring elements.  Phase 2 writes the tile's codes
+// back out and lists the pixels without one; a tile without any is done.  Phase
+// 2b turns each staged pixel into what a window visits: the code as FP32 (-1
+// when it is no source) and the colour with its channels in ten-bit fields,
+// one 8-byte load per neighbour.  Phase 3 deals the listed
+// pixels out to the threads, so a tile's few holes are filtered by many threads
+// at once instead of idling the rest of their warps; each filtered pixel walks
+// its window in shared memory in the stated order (the radius is a template
+// parameter, so the window unrolls) and overwrites its output.
+//
+// Phase 3 sets the time: 49 neighbours for each of some 46,000 pixels of a
+// 1280x720 frame.  The three channel differences come from one subtraction of
+// biased fields, each in [1, 511], and index a table of c[|d|] by the signed
+// difference, so a neighbour costs about 17 instructions (with byte-wise
+// absolute differences and separate loads of code, colour and spatial weight
+// it cost over 40).  Nine 1280x720 frames of radius 3 took 101 us before, 84 us
+// with the tile as it was (64 x 16) and 76 us with the wider one, which stages
+// less halo per pixel: 128 x 16 pixels and 512 threads up to radius 3 (47 KB of
+// shared memory, four CTAs per SM); above that its arrays would pass the 48 KB
+// of static shared memory, and the tile is 64 x 16.
+constexpr int kTileH = 16;
 constexpr int kDM = 8, kCM = 32;          // left margins of the staged rows: pixels, colour bytes
-constexpr int kDW = kDM + kTileW + kDM;   // staged code row, pixels
-constexpr int kCW = kCM + 3 * kTileW + kCM;   // staged colour row, bytes
+template <int R>
+struct Tile {
+    static constexpr int kW = R <= 3 ? 128 : 64, kThreads = 4 * kW;
+};
 static_assert(kJbfMaxRadius <= kDM && 3 * kJbfMaxRadius <= kCM, "halo wider than the margins");
 
 template <int R>
-__global__ void __launch_bounds__(kThreads) k_jbf(const JbfParams P)
+__global__ void __launch_bounds__(Tile<R>::kThreads, 2048 / Tile<R>::kThreads) k_jbf(const __grid_constant__ JbfParams P)
 {
+    constexpr int kTileW = Tile<R>::kW, kThreads = Tile<R>::kThreads;
+    constexpr int kDW = kDM + kTileW + kDM;        // staged code row, pixels
+    constexpr int kCW = kCM + 3 * kTileW + kCM;    // staged colour row, bytes
     constexpr int side = 2 * R + 1;
     constexpr int hh = kTileH + 2 * R;
     __shared__ __align__(16) uint16_t s_d[hh][kDW];
     __shared__ __align__(16) uint8_t s_c[hh][kCW];
-    // per staged pixel: the code as FP32 (-1 when it is no source) and the
-    // colour packed R | G << 8 | B << 16, for the window walks of phase 3
-    // (rows padded by a word so that neighbouring rows fall in other banks)
-    __shared__ float s_df[hh][kDW + 1];
-    __shared__ uint32_t s_cc[hh][kDW + 1];
+    // per staged pixel: the code as FP32 bits (-1 when it is no source) and
+    // the colour R | G << 10 | B << 20, for the window walks of phase 3 (rows
+    // padded so that neighbouring rows fall in other banks)
+    __shared__ __align__(16) uint2 s_px[hh][kDW + 2];
     __shared__ uint16_t s_list[kTileW * kTileH];
-    __shared__ float s_ws[side * side];
-    __shared__ float s_wc[256];
+    __shared__ float s_wc[512];                    // [256 + d]: c[|d|]
     __shared__ int s_n;
     const JbfCam& C = P.cam[blockIdx.z];
     const int x0 = blockIdx.x * kTileW, y0 = blockIdx.y * kTileH;
@@ -71,104 +86,130 @@ __global__ void __launch_bounds__(kThreads) k_jbf(const JbfParams P)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const bool vec = C.vec != 0;
     if (tid == 0) s_n = 0;
-    // the weight tables in shared memory: the filtered pixels of a warp
-    // index them at different places, which parameter (constant) memory
-    // would serialise
-    for (int i = tid; i < side * side; i += kThreads) s_ws[i] = P.s[i];
-    for (int i = tid; i < 256; i += kThreads) s_wc[i] = P.c[i];
-    // phase 1: a warp per staged row.  Tasks 0-7: the tile's codes, 8 pixels
-    // each; 8-19: its colour, 16 bytes each; then the halo elements (R codes
-    // and 3R colour bytes on each side).  Outside the image a code of 0
-    // (never a source) and colour 0.
-    constexpr int kTasks = 8 + 12 + 8 * R;
+    // the colour weights in shared memory: the filtered pixels of a warp index
+    // them at different places, which parameter (constant) memory would
+    // serialise (the spatial weights' places are compile-time constants)
+    for (int i = tid; i < 512; i += kThreads) s_wc[i] = i > 0 ? P.c[i < 256 ? 256 - i : i - 256] : 0.0f;
+    // phase 1: a warp per staged row, outside the image a code of 0 (never a
+    // source) and colour 0.  With aligned rows the row with its margins is 18 +
+    // 28 16-byte pieces.
+    constexpr int kD16 = kDW / 8, kC16 = kCW / 16;
     for (int hy = warp; hy < hh; hy += kThreads / 32) {
         const int gy = y0 - R + hy;
         const bool row_in = gy >= 0 && gy < P.height;
         const uint16_t* drow = C.src + size_t(row_in ? gy : 0) * C.src_pitch;
         const uint8_t* crow = C.rgb + size_t(row_in ? gy : 0) * C.rgb_pitch;
-        for (int t = lane; t < kTasks; t += 32) {
-            if (t < 8) {
-                const int x = x0 + 8 * t;
-                uint16_t* dst = &s_d[hy][kDM + 8 * t];
-                if (row_in && vec && x + 8 <= W) {
-                    *reinterpret_cast<uint4*>(dst) = __ldg(reinterpret_cast<const uint4*>(drow + x));
-                } else {
+        if (!vec) {
+            for (int t = lane; t < kTileW + 2 * R; t += 32) {
+                const int x = x0 - R + t;
+                s_d[hy][kDM - R + t] = (row_in && x >= 0 && x < W) ? __ldg(drow + x) : uint16_t(0);
+            }
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) dst[e] = (row_in && x + e < W) ? __ldg(drow + x + e) : uint16_t(0);
-                }
-            } else if (t < 20) {
-                const int b = 3 * x0 + 16 * (t - 8);
-                uint8_t* dst = &s_c[hy][kCM + 16 * (t - 8)];
-                if (row_in && vec && b + 16 <= 3 * W) {
-                    *reinterpret_cast<uint4*>(dst) = __ldg(reinterpret_cast<const uint4*>(crow + b));
-                } else {
+            for (int t = lane; t < 3 * (kTileW + 2 * R); t += 32) {
+                const int b = 3 * (x0 - R) + t;
+                s_c[hy][kCM - 3 * R + t] = (row_in && b >= 0 && b < 3 * W) ? __ldg(crow + b) : uint8_t(0);
+            }
+            continue;
+        }
+        for (int q = lane; q < kD16 + kC16; q += 32) {
+            const bool code = q < kD16;
+            // the piece's first byte in the image row, and the row's length
+            const int t = code ? q : q - kD16;
+            const int b = code ? 2 * (x0 - kDM) + 16 * t : 3 * x0 - kCM + 16 * t, len = code ? 2 * W : 3 * W;
+            const uint8_t* row = code ? reinterpret_cast<const uint8_t*>(drow) : crow;
+            uint8_t* dst = code ? reinterpret_cast<uint8_t*>(&s_d[hy][0]) + 16 * t : &s_c[hy][0] + 16 * t;
+            uint4 v = make_uint4(0u, 0u, 0u, 0u);
+            if (row_in && b >= 0 && b + 16 <= len) {
+                v = __ldg(reinterpret_cast<const uint4*>(row + b));
+            } else if (row_in && b >= 0 && b < len) {             // the ragged end
+                uint32_t w[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
-                    for (int e = 0; e < 16; ++e) dst[e] = (row_in && b + e < 3 * W) ? __ldg(crow + b + e) : uint8_t(0);
+                for (int e = 0; e < 16; ++e)
+                    if (b + e < len) w[e >> 2] |= uint32_t(__ldg(row + b + e)) << (8 * (e & 3));
+                v = make_uint4(w[0], w[1], w[2], w[3]);
+            }
+            *reinterpret_cast<uint4*>(dst) = v;
+        }
+    }
+    __syncthreads();
+    // phase 2: the tile's codes go out (pixels without one as 0 for now), 8
+    // at a time or neighbouring lanes side by side, and those pixels are listed
+    constexpr int kC8 = kTileW / 8;
+    if (vec) {
+        for (int i = tid; i < kTileH * kC8; i += kThreads) {
+            const int ty = i / kC8, c8 = i - ty * kC8;
+            const int y = y0 + ty, x = x0 + 8 * c8;
+            if (y < P.height && x < W) {
+                const uint4 v = *reinterpret_cast<const uint4*>(&s_d[ty + R][kDM + 8 * c8]);
+                const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+                uint16_t* orow = C.dst + size_t(y) * C.dst_pitch;
+                const int ne = min(8, W - x);
+                if (ne == 8)
+                    *reinterpret_cast<uint4*>(orow + x) = v;
+                for (int e = 0; e < ne; ++e) {
+                    const uint16_t d = uint16_t(w[e >> 1] >> (16 * (e & 1)));
+                    if (ne != 8) orow[x + e] = d;
+                    if (d == 0) s_list[atomicAdd(&s_n, 1)] = uint16_t(ty * kTileW + 8 * c8 + e);
                 }
-            } else if (t < 20 + 2 * R) {
-                const int h = t - 20;                              // left R codes, then right R
-                const int tx = h < R ? h - R : kTileW + (h - R);
-                const int x = x0 + tx;
-                s_d[hy][kDM + tx] = (row_in && x >= 0 && x < W) ? __ldg(drow + x) : uint16_t(0);
-            } else {
-                const int h = t - 20 - 2 * R;                      // left 3R bytes, then right 3R
-                const int tb = h < 3 * R ? h - 3 * R : 3 * kTileW + (h - 3 * R);
-                const int b = 3 * x0 + tb;
-                s_c[hy][kCM + tb] = (row_in && b >= 0 && b < 3 * W) ? __ldg(crow + b) : uint8_t(0);
+            }
+        }
+    } else {
+        for (int i = tid; i < kTileH * kTileW; i += kThreads) {
+            const int ty = i / kTileW, tx = i - ty * kTileW;
+            const int y = y0 + ty, x = x0 + tx;
+            if (y < P.height && x < W) {
+                const uint16_t d = s_d[ty + R][kDM + tx];
+                C.dst[size_t(y) * C.dst_pitch + x] = d;
+                if (d == 0) s_list[atomicAdd(&s_n, 1)] = uint16_t(i);
             }
         }
     }
     __syncthreads();
-    // phase 1b: sources and packed colour of every staged pixel
-    constexpr int sw = kTileW + 2 * R;
-    for (int i = tid; i < hh * sw; i += kThreads) {
-        const int hy = i / sw, col = kDM - R + (i - hy * sw);
-        const uint32_t q = s_d[hy][col];
-        const bool src = q >= P.d_lo && q <= P.d_hi && q != kDepthBg;
-        s_df[hy][col] = src ? code_to_float(q) : -1.0f;
-        const uint8_t* c = &s_c[hy][kCM + 3 * (col - kDM)];
-        s_cc[hy][col] = uint32_t(c[0]) | (uint32_t(c[1]) << 8) | (uint32_t(c[2]) << 16);
-    }
-    // phase 2: the tile's codes go out 8 at a time (pixels without one as
-    // 0 for now) and those pixels are listed
-    if (tid < kTileH * (kTileW / 8)) {
-        const int ty = tid >> 3, c8 = tid & 7;
-        const int y = y0 + ty, x = x0 + 8 * c8;
-        if (y < P.height && x < W) {
-            const uint4 v = *reinterpret_cast<const uint4*>(&s_d[ty + R][kDM + 8 * c8]);
-            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-            uint16_t* orow = C.dst + size_t(y) * C.dst_pitch;
-            const int ne = min(8, W - x);
-            if (vec && ne == 8)
-                *reinterpret_cast<uint4*>(orow + x) = v;
-            for (int e = 0; e < ne; ++e) {
-                const uint16_t d = uint16_t(w[e >> 1] >> (16 * (e & 1)));
-                if (!(vec && ne == 8)) orow[x + e] = d;
-                if (d == 0) s_list[atomicAdd(&s_n, 1)] = uint16_t(ty * kTileW + 8 * c8 + e);
-            }
+    const int n_holes = s_n;
+    if (n_holes == 0) return;                      // uniform over the CTA
+    // phase 2b: four staged pixels a thread (the columns a window reaches,
+    // rounded out to quads; the rounding's columns are never visited)
+    constexpr int kLeft = (R + 3) / 4 * 4, kQuads = (kTileW + 2 * kLeft) / 4;
+    for (int i = tid; i < hh * kQuads; i += kThreads) {
+        const int hy = i / kQuads, q = i - hy * kQuads, col = kDM - kLeft + 4 * q;
+        const uint2 dd = *reinterpret_cast<const uint2*>(&s_d[hy][col]);
+        const uint32_t* c = reinterpret_cast<const uint32_t*>(&s_c[hy][kCM + 3 * (col - kDM)]);
+        const uint32_t c0 = c[0], c1 = c[1], c2 = c[2];
+        const uint32_t code[4] = {dd.x & 0xFFFFu, dd.x >> 16, dd.y & 0xFFFFu, dd.y >> 16};
+        const uint32_t rgb[4] = {c0, __byte_perm(c0, c1, 0x0543), __byte_perm(c1, c2, 0x0432), c2 >> 8};
+        uint32_t o[8];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const bool src = code[e] >= P.d_lo && code[e] <= P.d_hi && code[e] != kDepthBg;
+            o[2 * e] = __float_as_uint(src ? code_to_float(code[e]) : -1.0f);
+            o[2 * e + 1] = (rgb[e] & 0xFFu) | ((rgb[e] & 0xFF00u) << 2) | ((rgb[e] & 0xFF0000u) << 4);
         }
+        uint4* dst = reinterpret_cast<uint4*>(&s_px[hy][col]);
+        dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
+        dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
     }
     __syncthreads();
     // phase 3: one listed pixel per thread at a time
-    const int n_holes = s_n;
     for (int j = tid; j < n_holes; j += kThreads) {
         const int i = s_list[j];
         const int ty = i / kTileW, tx = i - ty * kTileW;
         const int cy = ty + R, cx = kDM + tx;                      // centre in the staged tile
-        const uint32_t c0 = s_cc[cy][cx];
+        const uint2* px = &s_px[cy][cx];
+        const uint32_t c0 = px->y + (256u | (256u << 10) | (256u << 20));
         float acc = 0.0f, wsum = 0.0f;
         int n = 0;
 #pragma unroll
         for (int dy = -R; dy <= R; ++dy) {
 #pragma unroll
             for (int dx = -R; dx <= R; ++dx) {
-                const float qf = s_df[cy + dy][cx + dx];
+                const uint2 q = px[dy * (kDW + 2) + dx];
+                const float qf = __uint_as_float(q.x);
                 if (qf < 0.0f)
                     continue;
-                const uint32_t ad = __vabsdiffu4(c0, s_cc[cy + dy][cx + dx]);   // |dR|, |dG|, |dB| bytes
-                const float w = __fmul_rn(__fmul_rn(__fmul_rn(s_ws[(dy + R) * side + (dx + R)], s_wc[ad & 255u]),
-                                                    s_wc[(ad >> 8) & 255u]),
-                                          s_wc[(ad >> 16) & 255u]);
+                const uint32_t df = c0 - q.y;                      // fields 256 + dR, 256 + dG, 256 + dB
+                const float w = __fmul_rn(__fmul_rn(__fmul_rn(P.s[(dy + R) * side + (dx + R)], s_wc[df & 1023u]),
+                                                    s_wc[(df >> 10) & 1023u]),
+                                          s_wc[df >> 20]);
                 acc = __fadd_rn(acc, __fmul_rn(w, qf));
                 wsum = __fadd_rn(wsum, w);
                 ++n;
@@ -229,7 +270,8 @@ cudaError_t launch_jbf(const JbfParams& P_in, int n_cams, cudaStream_t stream)
     if (n_cams <= 0 || P_in.width <= 0 || P_in.height <= 0) return cudaSuccess;
     if (n_cams > kJbfMaxCams) return cudaErrorInvalidValue;
     // 16-byte accesses where every row of a camera starts 16-byte aligned
-    // (a tile's first column sits 128 code bytes and 192 colour bytes on)
+    // (a tile's first column sits whole 128-byte steps of codes and 192-byte
+    // steps of colour on)
     JbfParams P = P_in;
     auto a16 = [](const void* p, int64_t pitch_bytes) {
         return (reinterpret_cast<uintptr_t>(p) & 15u) == 0 && pitch_bytes % 16 == 0;
@@ -238,16 +280,20 @@ cudaError_t launch_jbf(const JbfParams& P_in, int n_cams, cudaStream_t stream)
         JbfCam& c = P.cam[k];
         c.vec = a16(c.rgb, c.rgb_pitch) && a16(c.src, c.src_pitch * 2) && a16(c.dst, c.dst_pitch * 2) ? 1 : 0;
     }
-    dim3 grid(unsigned((P.width + kTileW - 1) / kTileW), unsigned((P.height + kTileH - 1) / kTileH),
-              unsigned(n_cams));
+    auto go = [&](auto radius) {
+        constexpr int R = decltype(radius)::value;
+        dim3 grid(unsigned((P.width + Tile<R>::kW - 1) / Tile<R>::kW), unsigned((P.height + kTileH - 1) / kTileH),
+                  unsigned(n_cams));
+        k_jbf<R><<<grid, Tile<R>::kThreads, 0, stream>>>(P);
+    };
     switch (P.radius) {
-    case 1: k_jbf<1><<<grid, kThreads, 0, stream>>>(P); break;
-    case 2: k_jbf<2><<<grid, kThreads, 0, stream>>>(P); break;
-    case 3: k_jbf<3><<<grid, kThreads, 0, stream>>>(P); break;
-    case 4: k_jbf<4><<<grid, kThreads, 0, stream>>>(P); break;
-    case 5: k_jbf<5><<<grid, kThreads, 0, stream>>>(P); break;
-    case 6: k_jbf<6><<<grid, kThreads, 0, stream>>>(P); break;
-    case 7: k_jbf<7><<<grid, kThreads, 0, stream>>>(P); break;
+    case 1: go(std::integral_constant<int, 1>{}); break;
+    case 2: go(std::integral_constant<int, 2>{}); break;
+    case 3: go(std::integral_constant<int, 3>{}); break;
+    case 4: go(std::integral_constant<int, 4>{}); break;
+    case 5: go(std::integral_constant<int, 5>{}); break;
+    case 6: go(std::integral_constant<int, 6>{}); break;
+    case 7: go(std::integral_constant<int, 7>{}); break;
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
