@@ -3,8 +3,8 @@
 //
 // GEMM view: M = 128 consecutive output pixels of one image row, N = the
 // output channels, K = 9 taps x input channels.  A tile is R such rows
-// (R = 4 for 32 output channels, 2 for up to 64, else 1; the folded and
-// wide forms below use 2).  A persistent CTA
+// (R = 4 for 32 output channels, 2 for up to 64, else 1; the wide form
+// below uses 2).  A persistent CTA
 // (one per SM) walks the tiles.  Input channels are taken in groups of one
 // 64-byte row (32 bf16 or 64 e4m3 channels).  For each tile and group, ONE
 // TMA copy brings the halo -- rows y0-1..y0+R, pixels x0-1..x0+128, zero
@@ -13,15 +13,28 @@
 // swizzle.  Operand A of output row r and tap (ky, kx) is that same halo
 // seen through a descriptor whose start lies 130 (r + ky) + kx rows further
 // on: nine taps cost nine descriptors, not nine copies, and the halo's two
-// extra rows are shared by the R output rows (narrow layers are bound by
-// moving the halo).  The weights [cout][ky][kx][cin] stay
-// resident in shared memory when they fit; otherwise they stream through a
-// ring of one-ky slices (three taps).  The fp32 accumulators live in a TMEM
-// ring: the epilogue (scale, bias, ReLU, optional ReLU-derivative mask,
-// rounding to bf16 or e4m3, NHWC store -- staged through shared memory and
-// TMA where the output is strided or upsampled --, optional 2x2 max pooling
-// or 1x1 output head) drains tile i while the MMA thread accumulates the
-// next ones.
+// extra rows are shared by the R output rows.  The weights stay resident in
+// shared memory when they fit; otherwise they stream through a ring.  The
+// fp32 accumulators live in a TMEM ring: the epilogue (scale, bias, ReLU,
+// optional ReLU-derivative mask, rounding to bf16 or e4m3, NHWC store --
+// staged through shared memory and TMA where the output is strided or
+// upsampled --, optional 2x2 max pooling or 1x1 output head) drains tile i
+// while the MMA thread accumulates the next ones.
+//
+// Stacked taps (up to 64 output channels).  An MMA of M = 128, K = 16 takes
+// max(N / 2, (4096 + 32 N) / 128) cycles: its 4 KB of A and 32 N bytes of B
+// leave shared memory at 128 bytes a clock (measured 45, 48, 64, 128 cycles
+// at N = 32, 64, 128, 256).  With N = 32 four fifths of that is A, read again
+// for each of the three output rows that a halo row feeds.  So a halo row h
+// is multiplied once per (kx, K-step) by the taps of all ky it is needed for:
+// output row r = h - ky has its accumulator at column (R - 1 - r) kAcc, so
+// ascending ky is ascending columns, and one MMA of up to three taps' weights
+// stacked along N adds to up to three rows' accumulators.  Each accumulator
+// still sees its (ky, kx, K-step) products in that order, so the results are
+// those of nine separate MMAs to the bit.  The first product of a row, which
+// starts its accumulator afresh, is an MMA of its own.  With the MMAs issued by
+// a uniform warp (below), the bf16 forward of four 1280x720 views went from
+// 1385 to 1212 us.
 //
 // C8 (the first layer: 8 input features in 16 bytes per pixel, bf16, or 8
 // e4m3 codes and 8 zero bytes): the halo is copied as rows of 16 bytes, one
@@ -55,33 +68,39 @@ namespace {
 
 constexpr int kTileM = 128;
 constexpr int kRow = 64;                               // bytes of one pixel row of a channel group
-constexpr int kThreads = 320;
 constexpr int kMaxStages = 8;
 constexpr int kSmemLimit = 227 * 1024;
 constexpr int kHeader = 2048;                          // barriers (bytes 0..511) and bias (512..1279)
 constexpr int kSmemFixed = 1024 + kHeader;             // alignment slack + header
 
-// kFold (32 output channels, where a 128 x 32 MMA is bound by its issue
-// cost): the three kx taps of one ky run as ONE MMA of N = 96 against the
-// unshifted halo row, D[p][32 kx + c] = sum over ky of A_ky[p] W(ky, kx);
-// output pixel q is then D[q][c] + D[q+1][32+c] + D[q+2][64+c], summed in
-// the epilogue with warp shuffles.  Each TMEM lane quadrant (one epilogue
-// warp) holds its own window of 32 halo pixels, overlapping the next by 2,
-// so a warp finds all three terms of its first 30 pixels in its own lanes:
-// a tile covers 4 x 30 output pixels.
 // WIDE (96 and 128 output channels with streamed weights): two output rows
 // per tile instead of one, so that every weight slice streamed from L2 feeds
 // twice the MMAs.
-template <int COUT, bool FOLD = false, bool WIDE = false>
+// kStacked: the stacked-tap form (see the head of this file).
+// kFolded (32 output channels, two or more channel groups): the three kx taps
+// of one ky run as ONE MMA of N = 96 against the unshifted halo row,
+// D[p][32 kx + c] = sum over ky of A_ky[p] W(ky, kx); output pixel q is then
+// D[q][c] + D[q+1][32+c] + D[q+2][64+c], summed in the epilogue with warp
+// shuffles.  Each TMEM lane quadrant (one epilogue warp) holds its own window
+// of 32 halo pixels, overlapping the next by 2, so a warp finds all three terms
+// of its first 30 pixels in its own lanes: a tile covers 4 x 30 output pixels.
+// Two thirds of the stacked form's MMAs for a threefold TMEM read per tile, so
+// it pays from two channel groups on.
+enum Form { kPlain, kStacked, kFolded };
+
+template <int COUT, int FORM, bool WIDE = false>
 struct ConvCfg {
-    static_assert(!WIDE || (!FOLD && (COUT == 96 || COUT == 128)), "the wide form is for 96 or 128 channels");
-    static_assert(!FOLD || COUT == 32, "the folded form is for 32 output channels");
-    static constexpr bool kFold = FOLD;
-    static constexpr int kTap = COUT * kRow;           // B tile of one tap (COUT rows of 64 bytes)
-    static constexpr int kSlice = 3 * kTap;            // the three taps of one ky
-    static constexpr int kGroup = 9 * kTap;            // all taps of one channel group
-    static constexpr int kN = kFold ? 3 * COUT : COUT; // MMA N
+    static_assert(!WIDE || (FORM == kPlain && (COUT == 96 || COUT == 128)), "the wide form is for 96 or 128 channels");
+    static_assert(FORM != kStacked || COUT <= 64, "the stacked form is for up to 64 output channels");
+    static_assert(FORM != kFolded || COUT == 32, "the folded form is for 32 output channels");
+    static constexpr bool kStack = FORM == kStacked, kFold = FORM == kFolded;
+    static constexpr int kN = kFold ? 3 * COUT : COUT; // MMA N of the plain and folded forms
     static constexpr int kAcc = (kN + 31) / 32 * 32;   // TMEM columns of one output row's accumulator
+    static constexpr int kTapRows = kStack ? kAcc : COUT;  // B rows from one tap's weights to the next's
+    static constexpr int kTap = kTapRows * kRow;       // B tile of one tap (its COUT rows of 64 bytes)
+    static constexpr int kSlice = 3 * kTap;            // three taps: of one ky, or stacked: of one kx
+    static constexpr int kGroup = 9 * kTap;            // all taps of one channel group
+    static constexpr int kWRing = kStack ? kGroup : kSlice; // unit in which weights stream
     static constexpr int kRows = kFold ? 2 : WIDE ? 2 : COUT <= 32 ? 4 : COUT <= 64 ? 2 : 1;   // rows per tile
     static constexpr int kHaloPx = kFold ? 128 : kTileM + 2;           // halo pixels per halo row
     static constexpr int kQuad = kFold ? 30 : 32;      // output pixels per lane quadrant
@@ -93,9 +112,14 @@ struct ConvCfg {
     static constexpr int kHaloRows = kRows + 2;
     static constexpr int kHaloBytes = kHaloRows * kHaloPx * kRow;
     static constexpr int kHaloStage = (kHaloBytes + 1023) / 1024 * 1024;   // halo slot, 1024-aligned
-    // Output staging for the TMA stores: each of the eight epilogue warps
-    // owns a buffer of 32 pixels x one chunk of up to 64 channels,
-    // 1024-byte aligned (the 128-byte swizzle's period).
+    // accumulator column of output row r of a tile
+    __host__ __device__ static constexpr int col(int r) { return (kStack ? kRows - 1 - r : r) * kAcc; }
+    static constexpr int kGroups = 2;                  // epilogue groups
+    static constexpr int kEpiWarps = 4 * kGroups;
+    static constexpr int kThreads = 64 + 32 * kEpiWarps;
+    // Output staging for the TMA stores: each epilogue warp owns a buffer of
+    // 32 pixels x one chunk of up to 64 channels, 1024-byte aligned (the
+    // 128-byte swizzle's period).
     static constexpr int kChunk = COUT < 64 ? COUT : 64;
     __host__ __device__ static constexpr int out_buf(bool fp8) { return (32 * kChunk * (fp8 ? 1 : 2) + 1023) / 1024 * 1024; }
     static_assert(kTap % 1024 == 0, "tap tiles stay 1024-byte aligned");
@@ -108,15 +132,15 @@ struct Plan {
 
 // Shared memory: resident weights come first (they are read by every tile),
 // then the staged output, then the depth of the rings.  hs = 0: no plan fits.
-template <int COUT, bool FOLD, bool WIDE = false>
+template <int COUT, int FORM, bool WIDE = false>
 Plan make_plan(int groups, bool fp8, bool want_out)
 {
-    using C = ConvCfg<COUT, FOLD, WIDE>;
+    using C = ConvCfg<COUT, FORM, WIDE>;
     Plan p{};
     const int res = groups * C::kGroup;
     for (int out = want_out ? 2 : 0; out >= 0; --out) {
-        const int fixed = kSmemFixed + out * 8 * C::out_buf(fp8);
-        if (fixed + res + 3 * C::kHaloStage <= kSmemLimit) {
+        const int fixed = kSmemFixed + out * C::kEpiWarps * C::out_buf(fp8);
+        if (fixed + res + (out == 1 ? 2 : 3) * C::kHaloStage <= kSmemLimit) {
             p.resident = 1;
             p.out = out;
             p.hs = std::min(kMaxStages, (kSmemLimit - fixed - res) / C::kHaloStage);
@@ -125,15 +149,15 @@ Plan make_plan(int groups, bool fp8, bool want_out)
             return p;
         }
     }
-    for (int out = want_out ? 1 : 0; out >= 0; --out) {       // streamed: weight slices before staging
-        const int fixed = kSmemFixed + out * 8 * C::out_buf(fp8);
-        const int ws = std::min(kMaxStages, (kSmemLimit - fixed - 3 * C::kHaloStage) / C::kSlice);
+    for (int out = want_out ? 1 : 0; out >= 0; --out) {       // streamed: weights before staging
+        const int fixed = kSmemFixed + out * C::kEpiWarps * C::out_buf(fp8);
+        const int ws = std::min(kMaxStages, (kSmemLimit - fixed - 3 * C::kHaloStage) / C::kWRing);
         if (ws >= 2) {
             p.resident = 0;
             p.out = out;
             p.hs = 3;
             p.ws = ws;
-            p.smem = fixed + p.hs * C::kHaloStage + p.ws * C::kSlice;
+            p.smem = fixed + p.hs * C::kHaloStage + p.ws * C::kWRing;
             return p;
         }
     }
@@ -144,7 +168,7 @@ Plan make_plan(int groups, bool fp8, bool want_out)
 constexpr int kC8Px = 136;
 template <int COUT>
 struct C8Cfg {
-    static constexpr int kHaloRows = ConvCfg<COUT>::kHaloRows;
+    static constexpr int kHaloRows = ConvCfg<COUT, kPlain>::kHaloRows;
     static constexpr int kHaloBytes = kHaloRows * kC8Px * 16;
     static constexpr int kHaloStage = (kHaloBytes + 1023) / 1024 * 1024;
     static constexpr int kTap = COUT * 16;
@@ -157,7 +181,7 @@ Plan make_plan_c8(bool fp8, bool want_out)
     using C = C8Cfg<COUT>;
     Plan p{};
     for (int out = want_out ? 2 : 0; out >= 0; --out) {
-        const int fixed = kSmemFixed + out * 8 * ConvCfg<COUT>::out_buf(fp8);
+        const int fixed = kSmemFixed + out * ConvCfg<COUT, kPlain>::kEpiWarps * ConvCfg<COUT, kPlain>::out_buf(fp8);
         if (fixed + C::kWBytes + 2 * C::kHaloStage <= kSmemLimit) {
             p.resident = 1;
             p.out = out;
@@ -196,9 +220,9 @@ __device__ __forceinline__ uint32_t pack_e4m3x4(float a, float b, float c, float
 // field is +32 bytes (the second K-step).  Only the first MMA can start a
 // fresh accumulator (acc0 = 0).
 template <int COUT, bool FP8, int NKS>
-__device__ __forceinline__ void mma_row(uint32_t d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc0)
+__device__ __forceinline__ void mma_row(uint32_t d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc0, uint32_t lead)
 {
-    using Cfg = ConvCfg<COUT>;
+    using Cfg = ConvCfg<COUT, kPlain>;
 #pragma unroll
     for (int kx = 0; kx < 3; ++kx) {
 #pragma unroll
@@ -207,9 +231,9 @@ __device__ __forceinline__ void mma_row(uint32_t d, uint64_t da, uint64_t db, ui
             const uint64_t b = db + uint64_t((kx * Cfg::kTap) >> 4) + 2 * ks;
             const uint32_t acc = (kx | ks) != 0 ? 1u : acc0;
             if (FP8)
-                tc::mma_e4m3(d, a, b, idesc, acc);
+                tc::mma_e4m3_lead(d, a, b, idesc, acc, lead);
             else
-                tc::mma_bf16(d, a, b, idesc, acc);
+                tc::mma_bf16_lead(d, a, b, idesc, acc, lead);
         }
     }
 }
@@ -217,9 +241,9 @@ __device__ __forceinline__ void mma_row(uint32_t d, uint64_t da, uint64_t db, ui
 // All MMAs of one channel group with resident weights: taps (ky, kx), NKS
 // K-steps each, every descriptor offset a compile-time constant.
 template <int COUT, bool FP8, int NKS>
-__device__ __forceinline__ void mma_group(uint32_t d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc0)
+__device__ __forceinline__ void mma_group(uint32_t d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc0, uint32_t lead)
 {
-    using Cfg = ConvCfg<COUT>;
+    using Cfg = ConvCfg<COUT, kPlain>;
 #pragma unroll
     for (int ky = 0; ky < 3; ++ky)
 #pragma unroll
@@ -230,20 +254,57 @@ __device__ __forceinline__ void mma_group(uint32_t d, uint64_t da, uint64_t db, 
                 const uint64_t b = db + uint64_t((ky * Cfg::kSlice + kx * Cfg::kTap) >> 4) + 2 * ks;
                 const uint32_t acc = (ky | kx | ks) != 0 ? 1u : acc0;
                 if (FP8)
-                    tc::mma_e4m3(d, a, b, idesc, acc);
+                    tc::mma_e4m3_lead(d, a, b, idesc, acc, lead);
                 else
-                    tc::mma_bf16(d, a, b, idesc, acc);
+                    tc::mma_bf16_lead(d, a, b, idesc, acc, lead);
             }
 }
 
-// kFold: the MMAs of one output row and channel group, one per (ky, K-step)
+// The stacked MMAs of one channel group of a tile (see the head of this
+// file): halo rows in turn, kx, NKS K-steps of 32 bytes, every descriptor
+// offset a compile-time constant.  FIRST: the tile's first channel group,
+// whose first product of each output row starts that row's accumulator.
+template <int COUT, bool FP8, int NKS, bool FIRST>
+__device__ __forceinline__ void mma_stack(uint32_t d, uint64_t da, uint64_t db, uint32_t lead)
+{
+    using Cfg = ConvCfg<COUT, kStacked>;
+    constexpr int R = Cfg::kRows;
+    auto mma = [lead](uint32_t dd, uint64_t a, uint64_t b, int taps, uint32_t acc) {
+        const int n = (taps - 1) * Cfg::kAcc + COUT;
+        if (FP8)
+            tc::mma_e4m3_lead(dd, a, b, tc::idesc_e4m3(kTileM, n), acc, lead);
+        else
+            tc::mma_bf16_lead(dd, a, b, tc::idesc_bf16(kTileM, n), acc, lead);
+    };
+#pragma unroll
+    for (int h = 0; h < R + 2; ++h) {
+        // halo row h is row ky of the window of output row h - ky
+        const int lo = h >= R ? h - R + 1 : 0, hi = h < 2 ? h : 2, taps = hi - lo + 1;
+        const uint32_t dh = d + uint32_t(Cfg::col(h - lo));
+#pragma unroll
+        for (int kx = 0; kx < 3; ++kx)
+#pragma unroll
+            for (int ks = 0; ks < NKS; ++ks) {
+                const uint64_t a = da + uint64_t(((h * Cfg::kHaloPx + kx) * kRow) >> 4) + 2 * ks;
+                const uint64_t b = db + uint64_t((kx * Cfg::kSlice + lo * Cfg::kTap) >> 4) + 2 * ks;
+                if (FIRST && kx == 0 && ks == 0 && h < R) {
+                    mma(dh, a, b, 1, 0u);
+                    if (taps > 1) mma(dh + Cfg::kAcc, a, b + uint64_t(Cfg::kTap >> 4), taps - 1, 1u);
+                } else {
+                    mma(dh, a, b, taps, 1u);
+                }
+            }
+    }
+}
+
+// kFolded: the MMAs of one output row and channel group, one per (ky, K-step)
 // with N = 96; A of ky starts ky halo rows further on, B of ky is the
 // contiguous slice of its three taps.  NKY: slices resident (3, ky from the
 // group's base) or one streamed slice (1, the caller passes its ky's A).
 template <bool FP8, int NKS, int NKY>
-__device__ __forceinline__ void mma_fold(uint32_t d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc0)
+__device__ __forceinline__ void mma_fold(uint32_t d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc0, uint32_t lead)
 {
-    using Cfg = ConvCfg<32, true>;
+    using Cfg = ConvCfg<32, kFolded>;
 #pragma unroll
     for (int ky = 0; ky < NKY; ++ky)
 #pragma unroll
@@ -252,9 +313,9 @@ __device__ __forceinline__ void mma_fold(uint32_t d, uint64_t da, uint64_t db, u
             const uint64_t b = db + uint64_t((ky * Cfg::kSlice) >> 4) + 2 * ks;
             const uint32_t acc = (ky | ks) != 0 ? 1u : acc0;
             if (FP8)
-                tc::mma_e4m3(d, a, b, idesc, acc);
+                tc::mma_e4m3_lead(d, a, b, idesc, acc, lead);
             else
-                tc::mma_bf16(d, a, b, idesc, acc);
+                tc::mma_bf16_lead(d, a, b, idesc, acc, lead);
         }
 }
 
@@ -293,19 +354,20 @@ __device__ __forceinline__ uint32_t pool4_e4m3(const uint32_t (&c)[4])
 
 // FP8: e4m3 operands and output (K = 32 channels per MMA, 64 per group);
 // otherwise bf16 (K = 16, 32 per group).
-template <int COUT, bool FP8, bool FOLD, bool WIDE, bool C8>
-__global__ void __launch_bounds__(kThreads, 1)
+template <int COUT, bool FP8, int FORM, bool WIDE, bool C8>
+__global__ void __launch_bounds__(ConvCfg<COUT, FORM, WIDE>::kThreads, 1)
 k_conv3x3_tc(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CUtensorMap tmw,
              const __grid_constant__ CUtensorMap tmy, const __grid_constant__ CUtensorMap tmy2, ConvArgs P,
              int n_tiles, int HS, int WS, int resident, int tma_out)
 {
-    using Cfg = ConvCfg<COUT, FOLD, WIDE>;
-    static_assert(!C8 || (!FOLD && !WIDE && COUT <= 64), "the 16-byte-pixel form is for the first layer");
+    using Cfg = ConvCfg<COUT, FORM, WIDE>;
+    static_assert(!C8 || (FORM == kPlain && !WIDE && COUT <= 64), "the 16-byte-pixel form is for the first layer");
     // halo stage size and bytes per copy (C8: 16-byte pixel rows)
     constexpr int kStage = C8 ? C8Cfg<COUT>::kHaloStage : Cfg::kHaloStage;
     constexpr int kHaloTx = C8 ? C8Cfg<COUT>::kHaloBytes : Cfg::kHaloBytes;
     static_assert(512 + 4 * COUT <= kHeader, "bias fits the header");
     static_assert(COUT > 64 || 768 + 4 * (3 * COUT + 3) <= kHeader, "head weights fit the header");
+    constexpr int kThreads = Cfg::kThreads;
     constexpr int kPerGroup = FP8 ? 64 : 32;           // channels in one 64-byte row
     constexpr int kEsize = FP8 ? 1 : 2;
     constexpr int kOutBuf = Cfg::out_buf(FP8);
@@ -323,11 +385,11 @@ k_conv3x3_tc(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CU
     int* skip = reinterpret_cast<int*>(tmem_slot + 1);
     float* s_bias = reinterpret_cast<float*>(base + 512);          // [COUT] (<= 192 floats)
     float* s_head = reinterpret_cast<float*>(base + 768);          // fused head: [3][COUT] weights, [3] bias
-    uint8_t* sOut = base + kHeader;                                  // [8 warps][tma_out][kOutBuf]
-    uint8_t* sHalo = sOut + tma_out * 8 * kOutBuf;
+    uint8_t* sOut = base + kHeader;                                  // [kEpiWarps][tma_out][kOutBuf]
+    uint8_t* sHalo = sOut + tma_out * Cfg::kEpiWarps * kOutBuf;
     uint8_t* sW = sHalo + HS * kStage;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // (uniform)
     if (threadIdx.x == 0) *skip = *reinterpret_cast<volatile int*>(P.err);
     __syncthreads();
     if (*skip) return;                                 // an earlier CTA gave up
@@ -371,14 +433,24 @@ k_conv3x3_tc(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CU
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer
+        // stacked: the nine taps of channel group g, kx by kx (one copy of three
+        // taps where they are contiguous)
+        auto load_taps = [&](uint8_t* dst, uint64_t* bar, int g) {
+            for (int kx = 0; kx < 3; ++kx)
+                for (int ky = 0; ky < 3; ky += Cfg::kTapRows == COUT ? 3 : 1)
+                    tc::tma_load_4d(dst + kx * Cfg::kSlice + ky * Cfg::kTap, &tmw, bar, g * kPerGroup, 0, kx, ky);
+        };
         if (lane == 0) {
             if (C8) {
                 tc::mbar_arrive_expect_tx(wready, uint32_t(9 * C8Cfg<COUT>::kTap));
                 tc::tma_load_3d(sW, &tmw, wready, 0, 0, 0);
+            } else if (Cfg::kStack && resident) {
+                tc::mbar_arrive_expect_tx(wready, uint32_t(G * 9 * COUT * kRow));
+                for (int g = 0; g < G; ++g) load_taps(sW + g * Cfg::kGroup, wready, g);
             } else if (resident) {
                 tc::mbar_arrive_expect_tx(wready, uint32_t(G * Cfg::kGroup));
                 for (int g = 0; g < G; ++g)
@@ -412,7 +484,16 @@ k_conv3x3_tc(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CU
                         tc::tma_load_4d(sHalo + sh * kStage, &tmx, &full_h[sh], g * kPerGroup, x0 - 1, y0 - 1, n);
                     }
                     ++qh;
-                    if (!resident && !C8) {
+                    if (Cfg::kStack && !resident) {
+                        const int sw = int(qw % uint32_t(WS));
+                        if (!tc::mbar_wait_sleep(&empty_w[sw], ((qw / uint32_t(WS)) & 1u) ^ 1u, P.err, 2)) {
+                            ok = false;
+                            break;
+                        }
+                        tc::mbar_arrive_expect_tx(&full_w[sw], uint32_t(9 * COUT * kRow));
+                        load_taps(sW + sw * Cfg::kWRing, &full_w[sw], g);
+                        ++qw;
+                    } else if (!resident && !C8) {
                         for (int ky = 0; ky < 3; ++ky, ++qw) {
                             const int sw = int(qw % uint32_t(WS));
                             if (!tc::mbar_wait_sleep(&empty_w[sw], ((qw / uint32_t(WS)) & 1u) ^ 1u, P.err, 2)) {
@@ -431,17 +512,24 @@ k_conv3x3_tc(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CU
         // Ring slots and phase parities are running counters; every channel
         // group but the last holds two K-steps.  With resident weights a
         // group is one straight run of MMAs with compile-time descriptor
-        // offsets (the issue loop is the critical path of the kernel).
-        if (lane == 0) {
+        // offsets.  The whole warp runs this loop and lane 0 issues: the issue
+        // loop is the critical path of the kernel, and in a branch of one lane
+        // every descriptor is moved to uniform registers at its MMA, which made
+        // an MMA cost 74 to 111 cycles where the tensor cores take 45 to 64.
+        {
+            const uint32_t lead = lane == 0 ? 1u : 0u;
+            auto wait = [&](uint64_t* bar, uint32_t parity, int code) {
+                return __all_sync(0xffffffffu, tc::mbar_wait(bar, parity, P.err, code)) != 0;
+            };
             constexpr uint32_t idesc = FP8 ? tc::idesc_e4m3(kTileM, Cfg::kN) : tc::idesc_bf16(kTileM, Cfg::kN);
-            bool ok = (!resident && !C8) || tc::mbar_wait(wready, 0, P.err, 3);
+            bool ok = (!resident && !C8) || wait(wready, 0, 3);
             const int nks_last = (min(kPerGroup, Cin - (G - 1) * kPerGroup) * kEsize + 31) / 32;
             const uint64_t dh0 = tc::desc_kmajor_sw64(tc::smem_u32(sHalo));
             const uint64_t dw0 = tc::desc_kmajor_sw64(tc::smem_u32(sW));
             int sh = 0, sw = 0, b = 0;
             uint32_t ph = 0, pw = 0, pb = 0;
             for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
-                if (!tc::mbar_wait(&acc_empty[b], pb ^ 1u, P.err, 4)) {
+                if (!wait(&acc_empty[b], pb ^ 1u, 4)) {
                     ok = false;
                     break;
                 }
@@ -450,7 +538,7 @@ k_conv3x3_tc(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CU
                 for (int g = 0; g < G; ++g) {
                     // TMA completion on the mbarrier orders the halo for the tensor
                     // cores (both async proxy): no tcgen05 fence here
-                    if (!tc::mbar_wait(&full_h[sh], ph, P.err, 5)) {
+                    if (!wait(&full_h[sh], ph, 5)) {
                         ok = false;
                         break;
                     }
@@ -481,9 +569,36 @@ k_conv3x3_tc(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CU
 #pragma unroll
                             for (int i = 0; i < 5; ++i) {
                                 if (FP8)
-                                    tc::mma_e4m3(dr, a[i], bw[i], idesc, i != 0 ? 1u : acc0);
+                                    tc::mma_e4m3_lead(dr, a[i], bw[i], idesc, i != 0 ? 1u : acc0, lead);
                                 else
-                                    tc::mma_bf16(dr, a[i], bw[i], idesc, i != 0 ? 1u : acc0);
+                                    tc::mma_bf16_lead(dr, a[i], bw[i], idesc, i != 0 ? 1u : acc0, lead);
+                            }
+                        }
+                    } else if constexpr (Cfg::kStack) {
+                        uint64_t db = dw0 + uint64_t((g * Cfg::kGroup) >> 4);
+                        if (!resident) {
+                            if (!wait(&full_w[sw], pw, 6)) {
+                                ok = false;
+                                break;
+                            }
+                            db = dw0 + uint64_t((sw * Cfg::kWRing) >> 4);
+                        }
+                        if (g == 0) {
+                            if (two)
+                                mma_stack<COUT, FP8, 2, true>(d, da, db, lead);
+                            else
+                                mma_stack<COUT, FP8, 1, true>(d, da, db, lead);
+                        } else {
+                            if (two)
+                                mma_stack<COUT, FP8, 2, false>(d, da, db, lead);
+                            else
+                                mma_stack<COUT, FP8, 1, false>(d, da, db, lead);
+                        }
+                        if (!resident) {
+                            tc::mma_commit_lead(&empty_w[sw], lead);          // the weights are free once these finish
+                            if (++sw == WS) {
+                                sw = 0;
+                                pw ^= 1u;
                             }
                         }
                     } else if (resident) {
@@ -495,19 +610,19 @@ k_conv3x3_tc(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CU
                             const uint64_t dar = da + uint64_t((r * Cfg::kHaloPx * kRow) >> 4);
                             if constexpr (Cfg::kFold) {
                                 if (two)
-                                    mma_fold<FP8, 2, 3>(dr, dar, db, idesc, acc0);
+                                    mma_fold<FP8, 2, 3>(dr, dar, db, idesc, acc0, lead);
                                 else
-                                    mma_fold<FP8, 1, 3>(dr, dar, db, idesc, acc0);
+                                    mma_fold<FP8, 1, 3>(dr, dar, db, idesc, acc0, lead);
                             } else {
                                 if (two)
-                                    mma_group<COUT, FP8, 2>(dr, dar, db, idesc, acc0);
+                                    mma_group<COUT, FP8, 2>(dr, dar, db, idesc, acc0, lead);
                                 else
-                                    mma_group<COUT, FP8, 1>(dr, dar, db, idesc, acc0);
+                                    mma_group<COUT, FP8, 1>(dr, dar, db, idesc, acc0, lead);
                             }
                         }
                     } else {
                         for (int ky = 0; ky < 3; ++ky) {
-                            if (!tc::mbar_wait(&full_w[sw], pw, P.err, 6)) {
+                            if (!wait(&full_w[sw], pw, 6)) {
                                 ok = false;
                                 break;
                             }
@@ -519,17 +634,17 @@ k_conv3x3_tc(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CU
                                 const uint64_t dak = da + uint64_t(((r + ky) * Cfg::kHaloPx * kRow) >> 4);
                                 if constexpr (Cfg::kFold) {
                                     if (two)
-                                        mma_fold<FP8, 2, 1>(dr, dak, db, idesc, a0);
+                                        mma_fold<FP8, 2, 1>(dr, dak, db, idesc, a0, lead);
                                     else
-                                        mma_fold<FP8, 1, 1>(dr, dak, db, idesc, a0);
+                                        mma_fold<FP8, 1, 1>(dr, dak, db, idesc, a0, lead);
                                 } else {
                                     if (two)
-                                        mma_row<COUT, FP8, 2>(dr, dak, db, idesc, a0);
+                                        mma_row<COUT, FP8, 2>(dr, dak, db, idesc, a0, lead);
                                     else
-                                        mma_row<COUT, FP8, 1>(dr, dak, db, idesc, a0);
+                                        mma_row<COUT, FP8, 1>(dr, dak, db, idesc, a0, lead);
                                 }
                             }
-                            tc::mma_commit(&empty_w[sw]);      // the slice is free once these finish
+                            tc::mma_commit_lead(&empty_w[sw], lead);      // the slice is free once these finish
                             if (++sw == WS) {
                                 sw = 0;
                                 pw ^= 1u;
@@ -537,24 +652,24 @@ k_conv3x3_tc(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CU
                         }
                         if (!ok) break;
                     }
-                    tc::mma_commit(&empty_h[sh]);              // the halo slot is free once these finish
+                    tc::mma_commit_lead(&empty_h[sh], lead);              // the halo slot is free once these finish
                     if (++sh == HS) {
                         sh = 0;
                         ph ^= 1u;
                     }
                 }
                 if (!ok) break;
-                tc::mma_commit(&acc_full[b]);                  // the tile's accumulator is complete
+                tc::mma_commit_lead(&acc_full[b], lead);                  // the tile's accumulator is complete
                 if (++b == Cfg::kNumAcc) {
                     b = 0;
                     pb ^= 1u;
                 }
             }
-            tc::mma_commit(drain);                             // every issued MMA has finished
+            tc::mma_commit_lead(drain, lead);                             // every issued MMA has finished
         }
     } else {
         // ------------------------------------------------------------ epilogue
-        // Group eg = (w - 2) / 4 takes the tiles tl = eg, eg + 2, ... of this
+        // Group eg = (w - 2) / 4 takes the tiles tl = eg, eg + kGroups, ... of this
         // CTA.  Thread (warp w, lane l) owns output pixel x0 + 32 (w mod 4) + l
         // of each row; every lane runs the arithmetic (the shuffles of the
         // pooling need the whole warp) and only lanes inside the image load
@@ -575,7 +690,8 @@ k_conv3x3_tc(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CU
         for (int i = 0; i < kPoolW; ++i) ptop[i] = 0u;
         const bool ev = (lane & 1) == 0;
         int nst = 0;                                               // chunks this warp has staged
-        for (int tile = blockIdx.x + eg * gridDim.x, tl = eg; tile < n_tiles; tile += 2 * gridDim.x, tl += 2) {
+        for (int tile = blockIdx.x + eg * gridDim.x, tl = eg; tile < n_tiles;
+             tile += Cfg::kGroups * gridDim.x, tl += Cfg::kGroups) {
             const int b = tl % Cfg::kNumAcc;
             if (!tc::mbar_wait_sleep(&acc_full[b], (tl / Cfg::kNumAcc) & 1, P.err, 7)) break;
             tc::fence_after_sync();
@@ -602,7 +718,7 @@ k_conv3x3_tc(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CU
 #pragma unroll
                     for (int k = 0; k < 3; ++k) hrgb[k] = float(P.head_rgb[3 * p + k]);
                 }
-                const uint32_t taddr = tmem + (uint32_t(qd * 32) << 16) + uint32_t(b * Cfg::kTileAcc + rr * Cfg::kAcc);
+                const uint32_t taddr = tmem + (uint32_t(qd * 32) << 16) + uint32_t(b * Cfg::kTileAcc + Cfg::col(rr));
                 // up to 64 columns per TMEM round trip, in units of 16
 #pragma unroll 1
                 for (int c0 = 0; c0 < COUT; c0 += 64) {
@@ -879,6 +995,24 @@ cudaError_t make_weight_map(CUtensorMap* m, const void* w, int cout, int cin, bo
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
+// Stacked: w seen as (cin, cout, kx, ky); box {one channel group, cout, 1, ky
+// taps}: three taps of one kx where they are contiguous in shared memory, one
+// where they are padded apart
+cudaError_t make_weight_map_stack(CUtensorMap* m, const void* w, int cout, int cin, bool fp8, int taps)
+{
+    auto enc = encode_fn();
+    if (!enc) return cudaErrorNotSupported;
+    const cuuint64_t es = fp8 ? 1 : 2;
+    const cuuint64_t dims[4] = {cuuint64_t(cin), cuuint64_t(cout), 3, 3};
+    const cuuint64_t strides[3] = {cuuint64_t(9) * cin * es, cuuint64_t(cin) * es, cuuint64_t(3) * cin * es};
+    const cuuint32_t box[4] = {cuuint32_t(kRow / es), cuuint32_t(cout), 1, cuuint32_t(taps)};
+    const cuuint32_t el[4] = {1, 1, 1, 1};
+    CUresult r = enc(m, fp8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4,
+                     const_cast<void*>(w), dims, strides, box, el, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                     CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
 // C8: x [NB][H][W] pixels of 16 bytes (8 bf16 channels, or 16 e4m3 bytes),
 // halo box {16 bytes, kC8Px pixels, rows, 1 image}, no swizzle; quads (W a
 // multiple of 4): the same bytes as rows of four pixels, box {64 bytes,
@@ -967,7 +1101,7 @@ cudaError_t make_out_map(CUtensorMap* m, void* y, int NB, int H, int W, int ldy,
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-template <int COUT, bool FP8, bool FOLD = false, bool WIDE = false, bool C8 = false>
+template <int COUT, bool FP8, int FORM = (COUT <= 64 ? kStacked : kPlain), bool WIDE = false, bool C8 = false>
 cudaError_t launch_conv(const void* x, const void* w, ConvArgs a, cudaStream_t s)
 {
     constexpr int kPerGroup = FP8 ? 64 : 32;
@@ -976,17 +1110,19 @@ cudaError_t launch_conv(const void* x, const void* w, ConvArgs a, cudaStream_t s
     // channel slice of a wider tensor, or four times for the upsampling.  A
     // dense output is already written in whole lines by the threads.
     const bool want_out = a.up2 || a.ldy != COUT || a.coff != 0;
-    Plan p = C8 ? make_plan_c8<COUT>(FP8, want_out) : make_plan<COUT, FOLD, WIDE>(G, FP8, want_out);
+    Plan p = C8 ? make_plan_c8<COUT>(FP8, want_out) : make_plan<COUT, FORM, WIDE>(G, FP8, want_out);
     if (p.hs < 2 || (!p.resident && p.ws < 2)) return cudaErrorInvalidValue;
     CUtensorMap mx, mw, my, my2;
-    using C = ConvCfg<COUT, FOLD, WIDE>;
+    using C = ConvCfg<COUT, FORM, WIDE>;
     a.tiles_x = (a.W + C::kTileOut - 1) / C::kTileOut;
     a.x_quads = C8 && a.W % 4 == 0;
     cudaError_t e = C8         ? make_halo_map_c8(&mx, x, a.NB, a.H, a.W, FP8, C::kHaloRows, a.x_quads != 0)
                     : C::kFold ? make_halo_map(&mx, x, a.NB, a.H, a.W, a.xstride, FP8, 32, 1)
                                : make_halo_map(&mx, x, a.NB, a.H, a.W, a.xstride, FP8, C::kHaloPx, C::kHaloRows);
     if (e != cudaSuccess) return e;
-    e = C8 ? make_weight_map_c8(&mw, w, COUT, FP8) : make_weight_map(&mw, w, COUT, a.Cin, FP8);
+    e = C8          ? make_weight_map_c8(&mw, w, COUT, FP8)
+        : C::kStack ? make_weight_map_stack(&mw, w, COUT, a.Cin, FP8, C::kTapRows == COUT ? 3 : 1)
+                    : make_weight_map(&mw, w, COUT, a.Cin, FP8);
     if (e != cudaSuccess) return e;
     my = mw;                                           // unused unless the output maps are made
     my2 = mw;
@@ -999,13 +1135,13 @@ cudaError_t launch_conv(const void* x, const void* w, ConvArgs a, cudaStream_t s
                          cudaSuccess))
             p.out = 0;
     }
-    e = cudaFuncSetAttribute(k_conv3x3_tc<COUT, FP8, FOLD, WIDE, C8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    e = cudaFuncSetAttribute(k_conv3x3_tc<COUT, FP8, FORM, WIDE, C8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              p.smem);
     if (e != cudaSuccess) return e;
     const long long tiles = (long long)a.tiles_x * a.NB * ((a.H + C::kRows - 1) / C::kRows);
     const int grid = int(std::min<long long>(tiles, num_sms()));
-    k_conv3x3_tc<COUT, FP8, FOLD, WIDE, C8><<<grid, kThreads, p.smem, s>>>(mx, mw, my, my2, a, int(tiles), p.hs, p.ws,
-                                                                      p.resident, p.out);
+    k_conv3x3_tc<COUT, FP8, FORM, WIDE, C8><<<grid, C::kThreads, p.smem, s>>>(mx, mw, my, my2, a, int(tiles), p.hs, p.ws,
+                                                                         p.resident, p.out);
     return cudaGetLastError();
 }
 
@@ -1015,7 +1151,7 @@ bool streamed(const ConvArgs& a, bool fp8)
 {
     const int G = (a.Cin + (fp8 ? 64 : 32) - 1) / (fp8 ? 64 : 32);
     const bool want_out = a.up2 || (a.ldy && a.ldy != COUT) || a.coff != 0;
-    return !make_plan<COUT, false>(G, fp8, want_out).resident;
+    return !make_plan<COUT, kPlain>(G, fp8, want_out).resident;
 }
 
 template <bool FP8>
@@ -1025,22 +1161,22 @@ cudaError_t dispatch(const void* x, const void* w, int Cout, const ConvArgs& a, 
     const bool c8 = a.xstride * (FP8 ? 1 : 2) == 16;
     switch (Cout) {
     case 32:
-        if (c8) return launch_conv<32, FP8, false, false, true>(x, w, a, s);
+        if (c8) return launch_conv<32, FP8, kPlain, false, true>(x, w, a, s);
         // the folded form pays where the MMAs outweigh the epilogue: two or
         // more channel groups per tile.  It is kept to dense outputs without
         // the fused head (the network's uses of it)
         if (a.Cin > (FP8 ? 64 : 32) && !a.up2 && a.ldy == 32 && a.coff == 0 && !a.head_w)
-            return launch_conv<32, FP8, true>(x, w, a, s);
+            return launch_conv<32, FP8, kFolded>(x, w, a, s);
         return launch_conv<32, FP8>(x, w, a, s);
     case 48:
-        if (c8) return launch_conv<48, FP8, false, false, true>(x, w, a, s);
+        if (c8) return launch_conv<48, FP8, kPlain, false, true>(x, w, a, s);
         return launch_conv<48, FP8>(x, w, a, s);
     case 64: return launch_conv<64, FP8>(x, w, a, s);
     case 96:
-        if (streamed<96>(a, FP8)) return launch_conv<96, FP8, false, true>(x, w, a, s);
+        if (streamed<96>(a, FP8)) return launch_conv<96, FP8, kPlain, true>(x, w, a, s);
         return launch_conv<96, FP8>(x, w, a, s);
     case 128:
-        if (streamed<128>(a, FP8)) return launch_conv<128, FP8, false, true>(x, w, a, s);
+        if (streamed<128>(a, FP8)) return launch_conv<128, FP8, kPlain, true>(x, w, a, s);
         return launch_conv<128, FP8>(x, w, a, s);
     case 192: return launch_conv<192, FP8>(x, w, a, s);
     default: return cudaErrorInvalidValue;
