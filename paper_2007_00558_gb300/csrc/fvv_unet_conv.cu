@@ -47,10 +47,14 @@
 // TMA copy costs per row): the halo then starts at pixel x0 - 4, three
 // pixels before the window, and the descriptors start three pixels on.
 //
-// Warp roles (320 threads): 0 = TMA producer, 1 = TMEM owner and MMA issuer,
-// 2..9 = epilogue in two groups of four, taking alternate tiles (warp w
-// reads TMEM lanes 32 (w mod 4) .. +31); two warps per sub-partition hide
-// each other's TMEM-load and store latency.
+// Warp roles: 0 = TMA producer, 1 = TMEM owner and MMA issuer, the rest =
+// epilogue in groups of four (warp w reads TMEM lanes 32 (w mod 4) .. +31)
+// that take the tiles in turn: four groups at 32 channels, three at 48, else
+// two.  The epilogue is a chain of TMEM loads, arithmetic and stores per row,
+// so it takes several warps per scheduler to hide its latency: with four
+// groups for two, e1a of four 1280x720 views went from 87 to 71 us and d1b
+// from 141 to 113 us; at 64 channels three groups were slower (e2b 88 to
+// 106 us, the registers of a chunk spill).
 #include <algorithm>
 
 #include <cuda.h>
@@ -114,7 +118,9 @@ struct ConvCfg {
     static constexpr int kHaloStage = (kHaloBytes + 1023) / 1024 * 1024;   // halo slot, 1024-aligned
     // accumulator column of output row r of a tile
     __host__ __device__ static constexpr int col(int r) { return (kStack ? kRows - 1 - r : r) * kAcc; }
-    static constexpr int kGroups = 2;                  // epilogue groups
+    // epilogue groups: as many as a chunk's registers leave without spills (113,
+    // 146 and 200 a thread with four, three and two)
+    static constexpr int kGroups = kFold ? 2 : COUT <= 32 ? 4 : COUT <= 48 ? 3 : 2;
     static constexpr int kEpiWarps = 4 * kGroups;
     static constexpr int kThreads = 64 + 32 * kEpiWarps;
     // Output staging for the TMA stores: each epilogue warp owns a buffer of
@@ -206,6 +212,14 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b)
 {
     const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
     return *reinterpret_cast<const uint32_t*>(&h);
+}
+
+// max(0, .) of two bf16 values (a NaN gives 0, as fmaxf does)
+__device__ __forceinline__ uint32_t relu_bf16x2(uint32_t a)
+{
+    uint32_t r;
+    asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(0u));
+    return r;
 }
 
 __device__ __forceinline__ uint32_t pack_e4m3x4(float a, float b, float c, float d)
@@ -778,8 +792,14 @@ k_conv3x3_tc(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CU
                         const int c = c0 + 16 * u;
                         float v[16];
 #pragma unroll
-                        for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[u][j]) * P.acc_scale + s_bias[c + j];
-                        if (P.relu) {
+                        for (int j = 0; j < 16; j += 4) {
+                            const float4 bb = *reinterpret_cast<const float4*>(s_bias + c + j);
+                            v[j] = __uint_as_float(r[u][j]) * P.acc_scale + bb.x;
+                            v[j + 1] = __uint_as_float(r[u][j + 1]) * P.acc_scale + bb.y;
+                            v[j + 2] = __uint_as_float(r[u][j + 2]) * P.acc_scale + bb.z;
+                            v[j + 3] = __uint_as_float(r[u][j + 3]) * P.acc_scale + bb.w;
+                        }
+                        if (FP8 && P.relu) {
 #pragma unroll
                             for (int j = 0; j < 16; ++j) v[j] = fmaxf(v[j], 0.0f);
                         }
@@ -803,6 +823,12 @@ k_conv3x3_tc(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CU
                             }
 #pragma unroll
                             for (int m = 0; m < kW; ++m) w[m % kW] = pack_bf16x2(v[2 * m], v[2 * m + 1]);
+                            // the ReLU on the rounded pairs: rounding keeps signs and order, so
+                            // max(0, round(v)) = round(max(0, v)), at half the instructions
+                            if (P.relu) {
+#pragma unroll
+                                for (int m = 0; m < kW; ++m) w[m % kW] = relu_bf16x2(w[m % kW]);
+                            }
                         }
                         if constexpr (COUT <= 64) {
                             if (P.head_w) {
