@@ -45,16 +45,20 @@ __device__ __forceinline__ float code_to_float(uint32_t d)   // exact for d < 2^
 // its window in shared memory in the stated order (the radius is a template
 // parameter, so the window unrolls) and overwrites its output.
 //
-// Phase 3 sets the time: 49 neighbours for each of some 46,000 pixels of a
-// 1280x720 frame.  The three channel differences come from one subtraction of
-// biased fields, each in [1, 511], and index a table of c[|d|] by the signed
-// difference, so a neighbour costs about 17 instructions (with byte-wise
-// absolute differences and separate loads of code, colour and spatial weight
-// it cost over 40).  Nine 1280x720 frames of radius 3 took 101 us before, 84 us
-// with the tile as it was (64 x 16) and 76 us with the wider one, which stages
-// less halo per pixel: 128 x 16 pixels and 512 threads up to radius 3 (47 KB of
-// shared memory, four CTAs per SM); above that its arrays would pass the 48 KB
-// of static shared memory, and the tile is 64 x 16.
+// Latency sets the time: of the staging's loads, which a thread therefore has
+// all in flight together, and of phase 3, 49 neighbours in order for each of
+// some 46,000 pixels of a 1280x720 frame.  The three channel differences come
+// from one subtraction of biased fields, each in [1, 511], and index a table of
+// c[|d|] by the signed difference, so a neighbour costs about 17 instructions
+// (with byte-wise absolute differences and separate loads of code, colour and
+// spatial weight it cost over 40), and one that is no source adds zeros, so
+// that no branch keeps the next ones' loads back.  Nine 1280x720 frames of
+// radius 3 took 101 us before; 84 us with the cheaper neighbours, 76 us with
+// wider tiles, which stage less halo per pixel, 65 us without the branch and
+// 61 us with the staging's loads in flight.  Three CTAs per SM (40 registers)
+// take 67 us.  Tiles are 128 x 16 pixels for 512 threads up to radius 3 (47 KB
+// of shared memory, four CTAs per SM); above that the arrays would pass the 48
+// KB of static shared memory, and a tile is 64 x 16.
 constexpr int kTileH = 16;
 constexpr int kDM = 8, kCM = 32;          // left margins of the staged rows: pixels, colour bytes
 template <int R>
@@ -90,45 +94,61 @@ __global__ void __launch_bounds__(Tile<R>::kThreads, 2048 / Tile<R>::kThreads) k
     // them at different places, which parameter (constant) memory would
     // serialise (the spatial weights' places are compile-time constants)
     for (int i = tid; i < 512; i += kThreads) s_wc[i] = i > 0 ? P.c[i < 256 ? 256 - i : i - 256] : 0.0f;
-    // phase 1: a warp per staged row, outside the image a code of 0 (never a
-    // source) and colour 0.  With aligned rows the row with its margins is 18 +
-    // 28 16-byte pieces.
+    // phase 1: outside the image a code of 0 (never a source) and colour 0.
+    // With aligned rows a row with its margins is kD16 + kC16 16-byte pieces,
+    // dealt out over the threads; without, a warp takes a row.
     constexpr int kD16 = kDW / 8, kC16 = kCW / 16;
-    for (int hy = warp; hy < hh; hy += kThreads / 32) {
-        const int gy = y0 - R + hy;
-        const bool row_in = gy >= 0 && gy < P.height;
-        const uint16_t* drow = C.src + size_t(row_in ? gy : 0) * C.src_pitch;
-        const uint8_t* crow = C.rgb + size_t(row_in ? gy : 0) * C.rgb_pitch;
-        if (!vec) {
-            for (int t = lane; t < kTileW + 2 * R; t += 32) {
-                const int x = x0 - R + t;
-                s_d[hy][kDM - R + t] = (row_in && x >= 0 && x < W) ? __ldg(drow + x) : uint16_t(0);
-            }
+    if (vec) {
+        constexpr int kPieces = hh * (kD16 + kC16), kEach = (kPieces + kThreads - 1) / kThreads;
+        uint4 v[kEach];
 #pragma unroll
-            for (int t = lane; t < 3 * (kTileW + 2 * R); t += 32) {
-                const int b = 3 * (x0 - R) + t;
-                s_c[hy][kCM - 3 * R + t] = (row_in && b >= 0 && b < 3 * W) ? __ldg(crow + b) : uint8_t(0);
-            }
-            continue;
-        }
-        for (int q = lane; q < kD16 + kC16; q += 32) {
+        for (int e = 0; e < kEach; ++e) {                          // all of a thread's loads in flight together
+            const int i = tid + e * kThreads;
+            const int hy = i / (kD16 + kC16), q = i - hy * (kD16 + kC16), gy = y0 - R + hy;
             const bool code = q < kD16;
             // the piece's first byte in the image row, and the row's length
             const int t = code ? q : q - kD16;
             const int b = code ? 2 * (x0 - kDM) + 16 * t : 3 * x0 - kCM + 16 * t, len = code ? 2 * W : 3 * W;
-            const uint8_t* row = code ? reinterpret_cast<const uint8_t*>(drow) : crow;
-            uint8_t* dst = code ? reinterpret_cast<uint8_t*>(&s_d[hy][0]) + 16 * t : &s_c[hy][0] + 16 * t;
-            uint4 v = make_uint4(0u, 0u, 0u, 0u);
-            if (row_in && b >= 0 && b + 16 <= len) {
-                v = __ldg(reinterpret_cast<const uint4*>(row + b));
-            } else if (row_in && b >= 0 && b < len) {             // the ragged end
+            v[e] = make_uint4(0u, 0u, 0u, 0u);
+            if (i >= kPieces || gy < 0 || gy >= P.height || b < 0 || b >= len) continue;
+            const uint8_t* row = code ? reinterpret_cast<const uint8_t*>(C.src + size_t(gy) * C.src_pitch)
+                                      : C.rgb + size_t(gy) * C.rgb_pitch;
+            if (b + 16 <= len) {
+                v[e] = __ldg(reinterpret_cast<const uint4*>(row + b));
+            } else {                                               // the ragged end
                 uint32_t w[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
-                for (int e = 0; e < 16; ++e)
-                    if (b + e < len) w[e >> 2] |= uint32_t(__ldg(row + b + e)) << (8 * (e & 3));
-                v = make_uint4(w[0], w[1], w[2], w[3]);
+                for (int c = 0; c < 16; ++c)
+                    if (b + c < len) w[c >> 2] |= uint32_t(__ldg(row + b + c)) << (8 * (c & 3));
+                v[e] = make_uint4(w[0], w[1], w[2], w[3]);
             }
-            *reinterpret_cast<uint4*>(dst) = v;
+        }
+#pragma unroll
+        for (int e = 0; e < kEach; ++e) {
+            const int i = tid + e * kThreads;
+            if (i >= kPieces) break;
+            const int hy = i / (kD16 + kC16), q = i - hy * (kD16 + kC16);
+            uint8_t* dst = q < kD16 ? reinterpret_cast<uint8_t*>(&s_d[hy][0]) + 16 * q : &s_c[hy][0] + 16 * (q - kD16);
+            *reinterpret_cast<uint4*>(dst) = v[e];
+        }
+    } else {
+        for (int hy = warp; hy < hh; hy += kThreads / 32) {
+            const int gy = y0 - R + hy;
+            const bool row_in = gy >= 0 && gy < P.height;
+            const uint16_t* drow = C.src + size_t(row_in ? gy : 0) * C.src_pitch;
+            const uint8_t* crow = C.rgb + size_t(row_in ? gy : 0) * C.rgb_pitch;
+#pragma unroll
+            for (int t0 = 0; t0 < kTileW + 2 * R; t0 += 32) {
+                const int t = t0 + lane, x = x0 - R + t;
+                if (t < kTileW + 2 * R)
+                    s_d[hy][kDM - R + t] = (row_in && x >= 0 && x < W) ? __ldg(drow + x) : uint16_t(0);
+            }
+#pragma unroll
+            for (int t0 = 0; t0 < 3 * (kTileW + 2 * R); t0 += 32) {
+                const int t = t0 + lane, b = 3 * (x0 - R) + t;
+                if (t < 3 * (kTileW + 2 * R))
+                    s_c[hy][kCM - 3 * R + t] = (row_in && b >= 0 && b < 3 * W) ? __ldg(crow + b) : uint8_t(0);
+            }
         }
     }
     __syncthreads();
@@ -204,15 +224,14 @@ __global__ void __launch_bounds__(Tile<R>::kThreads, 2048 / Tile<R>::kThreads) k
             for (int dx = -R; dx <= R; ++dx) {
                 const uint2 q = px[dy * (kDW + 2) + dx];
                 const float qf = __uint_as_float(q.x);
-                if (qf < 0.0f)
-                    continue;
                 const uint32_t df = c0 - q.y;                      // fields 256 + dR, 256 + dG, 256 + dB
-                const float w = __fmul_rn(__fmul_rn(__fmul_rn(P.s[(dy + R) * side + (dx + R)], s_wc[df & 1023u]),
-                                                    s_wc[(df >> 10) & 1023u]),
-                                          s_wc[df >> 20]);
+                float w = __fmul_rn(__fmul_rn(__fmul_rn(P.s[(dy + R) * side + (dx + R)], s_wc[df & 1023u]),
+                                              s_wc[(df >> 10) & 1023u]),
+                                    s_wc[df >> 20]);
+                w = qf < 0.0f ? 0.0f : w;                          // no source: a zero more in each sum
                 acc = __fadd_rn(acc, __fmul_rn(w, qf));
                 wsum = __fadd_rn(wsum, w);
-                ++n;
+                n += qf < 0.0f ? 0 : 1;
             }
         }
         uint32_t out = 0u;
