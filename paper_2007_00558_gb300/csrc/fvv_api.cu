@@ -715,7 +715,7 @@ fvv_status fvv::run_batch(fvv_ctx* c, BatchScratch& S, int n, const fvv_view* vi
     std::vector<HostCopy> d2h;
     std::vector<std::pair<void*, const void*>> raw_copies;   // keys_raw
     std::vector<size_t> raw_bytes;
-    size_t koff = 0, soff = 0;
+    size_t koff = 0, soff = 0, points = 0;
     int max_chunks = 0;
     bool any_host = false;
     for (int i = 0; i < n; ++i) {
@@ -760,6 +760,9 @@ fvv_status fvv::run_batch(fvv_ctx* c, BatchScratch& S, int n, const fvv_view* vi
                 D.active[na] = k;
                 chunks += c->cams[k].height * ((c->cams[k].width + fvv::kSplatSeg - 1) / fvv::kSplatSeg);
                 D.chunk_begin[++na] = chunks;
+                points += size_t(c->cams[k].width) * c->cams[k].height;
+                D.eps = std::max(D.eps, fvv::map_eps(g[k], c->cams[k].width, c->cams[k].height, V.width, V.height,
+                                                     c->opt.z_min));
             }
         D.n_active = na;
         max_chunks = std::max(max_chunks, chunks);
@@ -819,7 +822,7 @@ fvv_status fvv::run_batch(fvv_ctx* c, BatchScratch& S, int n, const fvv_view* vi
         if (c->opt.layered || any_host || want_top3 || aux)
             return fail(FVV_ERR_INVALID_ARG, "persistent batches take device outputs and no aux outputs");
         int band = 1, sbx = 1;
-        fvv::persist_batch_shape(n, max_h, max_chunks, post->ctas, &band, &sbx);
+        fvv::persist_batch_shape(n, max_h, max_w, c->n_cams, post->max_width, max_chunks, post->ctas, &band, &sbx);
         post->batch = PersistBatch{vdev, c->frames_dev, S.keys, koff, n, max_h, band, sbx,
                                    c->opt.pixel_weights != 0 ? 1 : 0, {0, 0, 0}};
         post->slots.clear();
@@ -843,7 +846,7 @@ fvv_status fvv::run_batch(fvv_ctx* c, BatchScratch& S, int n, const fvv_view* vi
         FVV_CUDA(cudaMemcpyAsync(raw_copies[r].first, raw_copies[r].second, raw_bytes[r],
                                  cudaMemcpyDefault, s));
     FVV_TRY(run_kernel(c, kResolve, s, [&] {
-        return fvv::launch_resolve(vdev, n, max_h, max_w, c->n_cams, want_top3, c->frames_dev, s,
+        return fvv::launch_resolve(vdev, n, max_h, max_w, c->n_cams, points, want_top3, c->frames_dev, s,
                                    c->opt.layered != 0, c->opt.pixel_weights != 0);
     }));
     if (ahead) {

@@ -2,6 +2,7 @@
 // host runtime of libfvv.  Not part of the public ABI (see include/fvv.h).
 #pragma once
 
+#include <cmath>
 #include <cstddef>
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -15,7 +16,6 @@ constexpr uint16_t kDepthBg = 65535;   // depth code of a background pixel
 constexpr int kSplatSeg = 256;       // source pixels per splat warp (8 per lane, stride 32)
 constexpr int kSplatThreads = 256;
 constexpr int kResolveThreads = 256;
-constexpr int kResolveBand = 2;      // output rows per resolve CTA
 
 constexpr int kFlagCrack = 1;
 constexpr int kFlagFill = 2;
@@ -51,7 +51,7 @@ struct alignas(16) ViewDesc {
     int32_t flags;
     float tau_crack, tau_vis, z_min;
     uint32_t d_lo, d_hi;
-    int32_t pad0;
+    float eps;                       // tolerance of the division-free rounding: the largest map_eps of its cameras
     float vk[4];                     // the view's cx, cy, 1/fx, 1/fy (per-pixel weights)
     unsigned long long* keys;        // scratch z-buffer [Hv * Wv] (the FG layer when layered)
     unsigned long long* keys_bg;     // layered: the BG layer's z-buffer [Hv * Wv], else NULL
@@ -68,6 +68,44 @@ struct alignas(16) ViewDesc {
     int32_t active[kMaxCams];        // cameras with w > 0, ascending
     int32_t chunk_begin[kMaxCams + 1];  // prefix of splat warp segments over `active`
 };
+
+// Tolerance of the division-free rounding (fvv_kernels.cu, round_quotient2)
+// for quotients that matter below `dim` (the larger side of the target
+// image): half a last place below 2^ceil(log2 dim), and 2^-20 for the error
+// of the fraction and the one threshold off an exact half (at quotient 1/2).
+// m: the Z row of the map, applied to (x z, y z, z, 1) with x < W, y < H and
+// z up to zhi.  Infinite (every point by division) where images beyond 2^20
+// pixels a side leave the fraction too coarse, or where Z might leave the
+// range whose reciprocal is a normal number: above 2^100, or, unless z_min
+// keeps it off, nonzero below 2^-120 (Z is a multiple of its terms' last
+// places, so coefficients that are zero or at least 2^-70 rule that out).
+inline float settle_eps(int dim, float m0, float m1, float m2, float m3, float W, float H,
+                                            float zhi, float zmin)
+{
+    const float b0 = m0 < 0 ? -m0 : m0, b1 = m1 < 0 ? -m1 : m1, b2 = m2 < 0 ? -m2 : m2, b3 = m3 < 0 ? -m3 : m3;
+    const float big = (b0 * W + b1 * H + b2) * zhi + b3;
+    const float tiny = 8.4703295e-22f;                                   // 2^-70
+    const bool low = zmin < 7.8886091e-31f &&                            // 2^-100
+                     ((b0 != 0.0f && b0 < tiny) || (b1 != 0.0f && b1 < tiny) || (b2 != 0.0f && b2 < tiny) ||
+                      (b3 != 0.0f && b3 < tiny));
+    if (dim > (1 << 20) || !(big < 1.2676506e30f) || low) return HUGE_VALF;
+    int k = 0;
+    while ((1 << k) < dim) ++k;
+    return 2.9802322e-08f * float(1u << k) + 9.5367432e-07f;             // 2^(k - 25) + 2^-20
+}
+
+// Depths of view pixels for which a back-projection's tolerance holds: 2^-20
+// to 2^60 (pixels outside take the division).
+constexpr uint32_t kZNormLoBits = 0x35800000u, kZNormHiBits = 0x5D800000u;
+constexpr float kZNormHi = 1.152921504606847e18f;
+
+// That tolerance for both directions between a W x H camera and a Wv x Hv view.
+inline float map_eps(const CamGeom& G, int W, int H, int Wv, int Hv, float z_min)
+{
+    const float a = settle_eps(Wv > Hv ? Wv : Hv, G.M[8], G.M[9], G.M[10], G.M[11], float(W), float(H), 65536.0f, z_min);
+    const float b = settle_eps(W > H ? W : H, G.N[8], G.N[9], G.N[10], G.N[11], float(Wv), float(Hv), kZNormHi, z_min);
+    return a > b ? a : b;
+}
 
 // Persistent serving kernel (fvv_kernels.cu): one cooperative launch that
 // takes batches of views from a ring the host writes, and runs steps a-e of
@@ -105,8 +143,43 @@ cudaError_t launch_serve_persistent(PersistQueue* q_dev, PersistSync* sync, uint
                                     uint64_t idle_ns, uint64_t wait_ns, cudaStream_t stream, int* ctas);
 // The grid of that kernel for views up to max_w wide (0: none fits).
 int persist_grid(int max_w, int n_cams);
-// The band and the splat's CTAs per view the kernel uses for a batch.
-void persist_batch_shape(int n_views, int max_h, int max_chunks, int ctas, int* band, int* splat_bx);
+// The band and the splat's CTAs per view the kernel, launched for views up to
+// kernel_max_w wide, uses for a batch.
+void persist_batch_shape(int n_views, int max_h, int max_w, int n_cams, int kernel_max_w, int max_chunks, int ctas,
+                         int* band, int* splat_bx);
+
+// Programmatic dependent launch: a kernel launched with launch_behind may
+// start its CTAs once every CTA of the kernel before it on the stream has
+// called launch_dependents (or exited), and calls wait_primary, which returns
+// when that kernel is complete, before it touches memory.  What overlaps is
+// the launch itself: 1.5 us of the gap between two dependent kernels.
+#ifdef __CUDACC__
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_primary() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Both, at the head of a kernel that does nothing worth overlapping.
+__device__ __forceinline__ void behind()
+{
+    launch_dependents();
+    wait_primary();
+}
+
+template <class... P, class... A>
+cudaError_t launch_behind(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t stream, A... args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+#endif
 
 // Launchers (fvv_kernels.cu).  All asynchronous on `stream`.
 cudaError_t launch_clear_keys(unsigned long long* keys, size_t n, cudaStream_t stream);
@@ -115,7 +188,8 @@ cudaError_t launch_warp_splat(const ViewDesc* views, int n_views, int max_chunks
                               const FrameRef* frames, cudaStream_t stream, bool layered = false);
 // Layered: the crack filter of the BG layer (keys_bg -> keys_bgf), one pass.
 cudaError_t launch_crack_bg(const ViewDesc* views, int n_views, int max_h, int max_w, cudaStream_t stream);
-cudaError_t launch_resolve(const ViewDesc* views, int n_views, int max_h, int max_w, int n_cams,
+// points: the source pixels of all views' active cameras.
+cudaError_t launch_resolve(const ViewDesc* views, int n_views, int max_h, int max_w, int n_cams, size_t points,
                            bool top3, const FrameRef* frames, cudaStream_t stream, bool layered = false,
                            bool pixel_weights = false);
 cudaError_t launch_pack_rgba(const uint8_t* rgb, size_t rgb_pitch, uint32_t* rgba,

@@ -210,6 +210,7 @@ extern "C" fvv_status fvv_synthesize_noalloc(const fvv_rig* rig, const fvv_optio
     D.out_pitch = int64_t(out_pitch);
     D.geom = S.params->geom;                 // device addresses inside g_params
     int na = 0, segs = 0;
+    size_t points = 0;
     D.chunk_begin[0] = 0;
     for (int k = 0; k < nc; ++k) {
         fvv::FrameRef& F = P.frames[k];
@@ -223,6 +224,9 @@ extern "C" fvv_status fvv_synthesize_noalloc(const fvv_rig* rig, const fvv_optio
             D.active[na] = k;
             segs += F.H * ((F.W + fvv::kSplatSeg - 1) / fvv::kSplatSeg);
             D.chunk_begin[++na] = segs;
+            points += size_t(F.W) * F.H;
+            const float e = fvv::map_eps(P.geom[k], F.W, F.H, view->width, view->height, o.z_min);
+            if (!(e <= D.eps)) D.eps = e;
         }
     }
     D.n_active = na;
@@ -235,7 +239,8 @@ extern "C" fvv_status fvv_synthesize_noalloc(const fvv_rig* rig, const fvv_optio
     if (e == cudaSuccess) e = fvv::launch_clear_keys(S.keys, (np + 15) & ~size_t(15), s);
     if (e == cudaSuccess) e = fvv::launch_warp_splat(vdev, 1, segs, fdev, s);
     if (e == cudaSuccess)
-        e = fvv::launch_resolve(vdev, 1, view->height, view->width, nc, false, fdev, s, false, o.pixel_weights != 0);
+        e = fvv::launch_resolve(vdev, 1, view->height, view->width, nc, points, false, fdev, s, false,
+                                o.pixel_weights != 0);
     if (e != cudaSuccess) {
         cudaGetLastError();
         char msg[256];

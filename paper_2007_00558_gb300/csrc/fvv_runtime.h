@@ -291,6 +291,7 @@ size_t view_stage_bytes(const fvv_view& v, uint8_t* out_rgb, const fvv_aux* aux)
 // of launching (ctas: the kernel's grid, set by the caller).
 struct PersistPost {
     int ctas = 0;
+    int max_width = 1;                 // widest view the running kernel was launched for
     PersistBatch batch{};
     std::vector<int> slots;                    // frame-ring slots the batch reads
 };

@@ -382,6 +382,7 @@ fvv_status persist_submit(fvv_ctx* c, ServeState* st, ServeLane* L, const std::v
 {
     PersistPost P;
     P.ctas = st->pctas;
+    P.max_width = st->cfg.max_width;
     {
         std::lock_guard<std::recursive_mutex> g(c->mu);
         FVV_TRY(run_batch(c, L->S, int(views.size()), views.data(), nullptr, outs.data(), pitches.data(), nullptr,
