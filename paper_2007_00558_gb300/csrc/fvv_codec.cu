@@ -251,6 +251,51 @@ __global__ void __launch_bounds__(256) k_yuv_encode(const uint16_t* __restrict__
     v[size_t(by) * uvpitch + bx] = uint8_t(interleave4(p21 >> 8, p22 >> 8));
 }
 
+// The chroma byte of a 2x2 block's pixel pair from their 12-bit codes: the 4
+// MSBs spread to the even bits (two shift-and-mask steps), left and right.
+__device__ __forceinline__ uint32_t chroma_of(uint32_t left, uint32_t right)
+{
+    uint32_t m = (left >> 8) | (right & 0xF00u);        // left MSBs in bits 0-3, right in bits 8-11
+    m = (m | (m << 2)) & 0x3333u;
+    m = (m | (m << 1)) & 0x5555u;
+    return (m | (m >> 7)) & 0xFFu;
+}
+
+// 4 x 2 pixels (two 2x2 blocks) per thread: two 8-byte loads of codes, eight
+// lookups in flight together, 4-byte Y and 2-byte U and V stores.  A frame is
+// over in a few microseconds, so the latency of a load and a lookup and the
+// launch set the time; launches in a row overlap (launch_behind).  Encoding
+// nine 1280x720 frames and decoding them went from 53 to 45 us; with twice the
+// pixels a thread, so half the warps, it took 61 us.
+__global__ void __launch_bounds__(128) k_yuv_encode4(const uint16_t* __restrict__ depth, size_t dpitch, int groups,
+                                                     int bh, const uint16_t* __restrict__ lut, uint8_t* __restrict__ y,
+                                                     size_t ypitch, uint8_t* __restrict__ u, uint8_t* __restrict__ v,
+                                                     size_t uvpitch)
+{
+    launch_dependents();
+    const int i = blockIdx.x * 128 + threadIdx.x;
+    const int by = i / groups, g = i - by * groups;
+    wait_primary();
+    if (by >= bh) return;
+    uint2 q[2];
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+        q[r] = __ldg(reinterpret_cast<const uint2*>(reinterpret_cast<const uint8_t*>(depth) +
+                                                    size_t(2 * by + r) * dpitch + 8 * size_t(g)));
+    uint32_t c[2][4];
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) c[r][e] = __ldg(lut + (((e >> 1 ? q[r].y : q[r].x) >> (16 * (e & 1))) & 0xFFFFu));
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        const uint32_t yy = fold(c[r][0]) | (fold(c[r][1]) << 8) | (fold(c[r][2]) << 16) | (fold(c[r][3]) << 24);
+        const uint32_t cc = chroma_of(c[r][0], c[r][1]) | (chroma_of(c[r][2], c[r][3]) << 8);
+        *reinterpret_cast<uint32_t*>(y + size_t(2 * by + r) * ypitch + 4 * size_t(g)) = yy;
+        *reinterpret_cast<uint16_t*>((r ? v : u) + size_t(by) * uvpitch + 2 * size_t(g)) = uint16_t(cc);
+    }
+}
+
 bool on_dev(const void* p) { return p && mem_kind(p) == MemKind::Device; }
 
 fvv_status check_cam(fvv_ctx* c, int32_t cam)
@@ -377,6 +422,14 @@ fvv_status fvv_depth_encode_yuv(fvv_ctx* c, int32_t cam, const uint16_t* depth, 
     cudaStream_t s = stream ? static_cast<cudaStream_t>(stream) : c->own;
     const int bw = W / 2, bh = H / 2;
     const size_t n = size_t(bw) * bh;
+    // the wide form where every access it makes is aligned (45 us for 53 in the
+    // case above), else one 2x2 block a thread with accesses of its own width
+    if (W % 4 == 0 && fvv::aligned(depth, 8) && depth_pitch % 8 == 0 && fvv::aligned(y, 4) && y_pitch % 4 == 0 &&
+        fvv::aligned(u, 2) && fvv::aligned(v, 2) && uv_pitch % 2 == 0) {
+        FVV_CUDA(fvv::launch_behind(fvv::k_yuv_encode4, dim3(unsigned((n / 2 + 127) / 128)), 128, 0, s, depth, depth_pitch,
+                                    W / 4, bh, c->codec->enc[cam], y, y_pitch, u, v, uv_pitch));
+        return FVV_OK;
+    }
     fvv::k_yuv_encode<<<unsigned((n + 255) / 256), 256, 0, s>>>(depth, depth_pitch, bw, bh, c->codec->enc[cam], y,
                                                                y_pitch, u, v, uv_pitch);
     FVV_CUDA(cudaGetLastError());
