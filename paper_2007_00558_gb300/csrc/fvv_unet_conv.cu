@@ -403,6 +403,7 @@ k_conv3x3_tc(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CU
     uint8_t* sHalo = sOut + tma_out * Cfg::kEpiWarps * kOutBuf;
     uint8_t* sW = sHalo + HS * kStage;
 
+    behind();
     const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // (uniform)
     if (threadIdx.x == 0) *skip = *reinterpret_cast<volatile int*>(P.err);
     __syncthreads();
@@ -1166,9 +1167,8 @@ cudaError_t launch_conv(const void* x, const void* w, ConvArgs a, cudaStream_t s
     if (e != cudaSuccess) return e;
     const long long tiles = (long long)a.tiles_x * a.NB * ((a.H + C::kRows - 1) / C::kRows);
     const int grid = int(std::min<long long>(tiles, num_sms()));
-    k_conv3x3_tc<COUT, FP8, FORM, WIDE, C8><<<grid, C::kThreads, p.smem, s>>>(mx, mw, my, my2, a, int(tiles), p.hs, p.ws,
-                                                                         p.resident, p.out);
-    return cudaGetLastError();
+    return launch_behind(k_conv3x3_tc<COUT, FP8, FORM, WIDE, C8>, dim3(unsigned(grid)), C::kThreads, size_t(p.smem), s, mx,
+                         mw, my, my2, a, int(tiles), p.hs, p.ws, p.resident, p.out);
 }
 
 // Whether the one-row plan of a layer streams its weights.

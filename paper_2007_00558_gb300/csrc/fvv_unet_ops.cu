@@ -40,6 +40,7 @@ __global__ void k_pack_features(size_t npx, const uint8_t* __restrict__ rgb, con
                                 const uint8_t* __restrict__ hole, const float* __restrict__ top3, float inv_zfar,
                                 __nv_bfloat16* __restrict__ out)
 {
+    behind();
     const size_t p = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
     if (p >= npx) return;
     float f[8];
@@ -58,6 +59,7 @@ __global__ void k_pack_features_e4m3(size_t npx, const uint8_t* __restrict__ rgb
                                      const uint8_t* __restrict__ hole, const float* __restrict__ top3,
                                      float inv_zfar, float inv_s0, uint8_t* __restrict__ out)
 {
+    behind();
     const size_t p = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
     if (p >= npx) return;
     float f[8];
@@ -106,6 +108,7 @@ __device__ __forceinline__ void st8(__nv_bfloat16* p, const uint4 v) { *reinterp
 __global__ void k_maxpool2(int B, int H, int W, int C, const __nv_bfloat16* __restrict__ x, int ldx,
                            __nv_bfloat16* __restrict__ y, uint8_t* __restrict__ arg)
 {
+    behind();
     const size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
     const int h2 = H / 2, w2 = W / 2, cv = C >> 3;
     const size_t n_out = size_t(B) * h2 * w2 * cv;
@@ -146,6 +149,7 @@ __global__ void k_maxpool2_bwd(int B, int H, int W, int C, const __nv_bfloat16* 
                                const uint8_t* __restrict__ arg, const __nv_bfloat16* __restrict__ add,
                                const __nv_bfloat16* __restrict__ mask, int ldm, __nv_bfloat16* __restrict__ dx)
 {
+    behind();
     const size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
     const int cv = C >> 3;
     const size_t n = size_t(B) * H * W * cv;
@@ -183,6 +187,7 @@ __global__ void k_up2_concat_bwd(int B, int H, int W, int C1, int C2, const __nv
                                  const __nv_bfloat16* __restrict__ up_act, int ldu, __nv_bfloat16* __restrict__ dlo,
                                  __nv_bfloat16* __restrict__ dskip)
 {
+    behind();
     const int C = C1 + C2, cv1 = C1 >> 3, cv2 = C2 >> 3;
     const size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
     const int h2 = H / 2, w2 = W / 2;
@@ -226,6 +231,7 @@ __device__ __forceinline__ float e4m3_val(uint8_t b)
 __global__ void k_maxpool2_e4m3(int B, int H, int W, int C, const uint8_t* __restrict__ x, int ldx,
                                 uint8_t* __restrict__ y)
 {
+    behind();
     const size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
     const int h2 = H / 2, w2 = W / 2, cv = C >> 4;
     const size_t n_out = size_t(B) * h2 * w2 * cv;
@@ -292,6 +298,7 @@ __global__ void k_head_fwd(size_t npx, const T* __restrict__ d1, float s_d1, con
                            const float* __restrict__ bout, const uint8_t* __restrict__ rgb, float* __restrict__ s,
                            uint8_t* __restrict__ out, int W, size_t out_pitch, float* __restrict__ out_f32)
 {
+    behind();
     __shared__ float sw[3 * C1 + 3];
     for (int i = threadIdx.x; i < 3 * C1 + 3; i += blockDim.x) sw[i] = i < 3 * C1 ? wout[i] : bout[i - 3 * C1];
     __syncthreads();
@@ -330,6 +337,7 @@ __global__ void __launch_bounds__(128) k_head_bwd(size_t npx, const __nv_bfloat1
                                                   const uint8_t* __restrict__ target, float inv_count, size_t ppw,
                                                   float* __restrict__ part, __nv_bfloat16* __restrict__ dd1)
 {
+    behind();
     constexpr int KPL = (C1 + 31) / 32;                 // d1 channels per lane
     __shared__ float sw[3 * C1];
     for (int i = threadIdx.x; i < 3 * C1; i += blockDim.x) sw[i] = wout[i];
@@ -409,6 +417,7 @@ __global__ void __launch_bounds__(128) k_head_bwd(size_t npx, const __nv_bfloat1
 __global__ void __launch_bounds__(256) k_sum_splits(const float* __restrict__ part, int splits, size_t n,
                                                     float* out0, size_t n0, float* out1, size_t n1, float* out2)
 {
+    behind();
     __shared__ float red[8][32];
     const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
     const size_t i = size_t(blockIdx.x) * 32 + lane;
@@ -435,6 +444,7 @@ __global__ void __launch_bounds__(256) k_sum_splits(const float* __restrict__ pa
 __global__ void k_flip_weights(int Cout, int Cin, const float* __restrict__ w, __nv_bfloat16* __restrict__ wbf,
                                __nv_bfloat16* __restrict__ wt)
 {
+    behind();
     const size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
     const size_t n = size_t(Cout) * 9 * Cin;
     if (i >= n) return;
@@ -452,6 +462,7 @@ __global__ void k_flip_weights(int Cout, int Cin, const float* __restrict__ w, _
 // off[k] <= e < off[k + 1].
 __global__ void k_adam_multi(AdamList L, float lr, float b1, float b2, float eps, float c1, float c2)
 {
+    behind();
     const size_t stride = size_t(gridDim.x) * blockDim.x;
     for (size_t e = size_t(blockIdx.x) * blockDim.x + threadIdx.x; e < L.off[L.count]; e += stride) {
         int lo = 0, hi = L.count - 1;                    // the last k with off[k] <= e
@@ -483,6 +494,7 @@ __global__ void k_adam_multi(AdamList L, float lr, float b1, float b2, float eps
 // (out >= 0 on entry; non-negative floats order like their bits)
 __global__ void k_amax(size_t npix, int C, const __nv_bfloat16* __restrict__ x, int ld, float* __restrict__ out)
 {
+    behind();
     const int cv = C >> 3;
     const size_t n8 = npix * cv;
     float m = 0.0f;
@@ -503,7 +515,7 @@ unsigned blocks(size_t n, int t) { return unsigned((n + t - 1) / t); }
 cudaError_t launch_pack_features(size_t npx, const uint8_t* rgb, const float* depth, const uint8_t* hole,
                                  const float* top3, float z_far, __nv_bfloat16* out, cudaStream_t s)
 {
-    k_pack_features<<<blocks(npx, 256), 256, 0, s>>>(npx, rgb, depth, hole, top3, 1.0f / z_far, out);
+    launch_behind(k_pack_features, dim3(blocks(npx, 256)), 256, 0, s, npx, rgb, depth, hole, top3, 1.0f / z_far, out);
     return cudaGetLastError();
 }
 
@@ -511,7 +523,7 @@ cudaError_t launch_maxpool2(int B, int H, int W, int C, const __nv_bfloat16* x, 
                             uint8_t* arg, cudaStream_t s)
 {
     const size_t n = size_t(B) * (H / 2) * (W / 2) * (C / 8);
-    k_maxpool2<<<blocks(n, 256), 256, 0, s>>>(B, H, W, C, x, ldx, y, arg);
+    launch_behind(k_maxpool2, dim3(blocks(n, 256)), 256, 0, s, B, H, W, C, x, ldx, y, arg);
     return cudaGetLastError();
 }
 
@@ -520,7 +532,7 @@ cudaError_t launch_maxpool2_bwd(int B, int H, int W, int C, const __nv_bfloat16*
                                 cudaStream_t s)
 {
     const size_t n = size_t(B) * H * W * (C / 8);
-    k_maxpool2_bwd<<<blocks(n, 256), 256, 0, s>>>(B, H, W, C, dy, arg, add, mask, ldm, dx);
+    launch_behind(k_maxpool2_bwd, dim3(blocks(n, 256)), 256, 0, s, B, H, W, C, dy, arg, add, mask, ldm, dx);
     return cudaGetLastError();
 }
 
@@ -530,7 +542,7 @@ cudaError_t launch_up2_concat_bwd(int B, int H, int W, int C1, int C2, const __n
 {
     const size_t n_sk = size_t(B) * H * W * (C2 / 8), n_lo = size_t(B) * (H / 2) * (W / 2) * (C1 / 8);
     const size_t n = n_sk > n_lo ? n_sk : n_lo;
-    k_up2_concat_bwd<<<blocks(n, 256), 256, 0, s>>>(B, H, W, C1, C2, dcat, up_act, ldu, dlo, dskip);
+    launch_behind(k_up2_concat_bwd, dim3(blocks(n, 256)), 256, 0, s, B, H, W, C1, C2, dcat, up_act, ldu, dlo, dskip);
     return cudaGetLastError();
 }
 
@@ -541,9 +553,9 @@ cudaError_t launch_head_fwd(size_t npx, int C1, const __nv_bfloat16* d1, const f
                             float* out_f32, cudaStream_t s)
 {
     switch (C1) {
-    case 32: k_head_fwd<32><<<blocks(npx, 128), 128, 0, s>>>(npx, d1, 1.0f, wout, bout, rgb, sbuf, out, W, out_pitch, out_f32); break;
-    case 48: k_head_fwd<48><<<blocks(npx, 128), 128, 0, s>>>(npx, d1, 1.0f, wout, bout, rgb, sbuf, out, W, out_pitch, out_f32); break;
-    case 64: k_head_fwd<64><<<blocks(npx, 128), 128, 0, s>>>(npx, d1, 1.0f, wout, bout, rgb, sbuf, out, W, out_pitch, out_f32); break;
+    case 32: launch_behind(k_head_fwd<32, __nv_bfloat16>, dim3(blocks(npx, 128)), 128, 0, s, npx, d1, 1.0f, wout, bout, rgb, sbuf, out, W, out_pitch, out_f32); break;
+    case 48: launch_behind(k_head_fwd<48, __nv_bfloat16>, dim3(blocks(npx, 128)), 128, 0, s, npx, d1, 1.0f, wout, bout, rgb, sbuf, out, W, out_pitch, out_f32); break;
+    case 64: launch_behind(k_head_fwd<64, __nv_bfloat16>, dim3(blocks(npx, 128)), 128, 0, s, npx, d1, 1.0f, wout, bout, rgb, sbuf, out, W, out_pitch, out_f32); break;
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
@@ -554,9 +566,9 @@ cudaError_t launch_head_fwd_e4m3(size_t npx, int C1, const uint8_t* d1, float s_
                                  float* out_f32, cudaStream_t s)
 {
     switch (C1) {
-    case 32: k_head_fwd<32><<<blocks(npx, 128), 128, 0, s>>>(npx, d1, s_d1, wout, bout, rgb, nullptr, out, W, out_pitch, out_f32); break;
-    case 48: k_head_fwd<48><<<blocks(npx, 128), 128, 0, s>>>(npx, d1, s_d1, wout, bout, rgb, nullptr, out, W, out_pitch, out_f32); break;
-    case 64: k_head_fwd<64><<<blocks(npx, 128), 128, 0, s>>>(npx, d1, s_d1, wout, bout, rgb, nullptr, out, W, out_pitch, out_f32); break;
+    case 32: launch_behind(k_head_fwd<32, uint8_t>, dim3(blocks(npx, 128)), 128, 0, s, npx, d1, s_d1, wout, bout, rgb, nullptr, out, W, out_pitch, out_f32); break;
+    case 48: launch_behind(k_head_fwd<48, uint8_t>, dim3(blocks(npx, 128)), 128, 0, s, npx, d1, s_d1, wout, bout, rgb, nullptr, out, W, out_pitch, out_f32); break;
+    case 64: launch_behind(k_head_fwd<64, uint8_t>, dim3(blocks(npx, 128)), 128, 0, s, npx, d1, s_d1, wout, bout, rgb, nullptr, out, W, out_pitch, out_f32); break;
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
@@ -578,9 +590,9 @@ cudaError_t launch_head_bwd(size_t npx, int C1, const __nv_bfloat16* d1, const f
     const size_t nwarps = (npx + ppw - 1) / ppw;
     const unsigned grid = unsigned((nwarps + 3) / 4);
     switch (C1) {
-    case 32: k_head_bwd<32><<<grid, 128, 0, s>>>(npx, d1, wout, sbuf, target, inv, ppw, scratch, dd1); break;
-    case 48: k_head_bwd<48><<<grid, 128, 0, s>>>(npx, d1, wout, sbuf, target, inv, ppw, scratch, dd1); break;
-    case 64: k_head_bwd<64><<<grid, 128, 0, s>>>(npx, d1, wout, sbuf, target, inv, ppw, scratch, dd1); break;
+    case 32: launch_behind(k_head_bwd<32>, dim3(grid), 128, 0, s, npx, d1, wout, sbuf, target, inv, ppw, scratch, dd1); break;
+    case 48: launch_behind(k_head_bwd<48>, dim3(grid), 128, 0, s, npx, d1, wout, sbuf, target, inv, ppw, scratch, dd1); break;
+    case 64: launch_behind(k_head_bwd<64>, dim3(grid), 128, 0, s, npx, d1, wout, sbuf, target, inv, ppw, scratch, dd1); break;
     default: return cudaErrorInvalidValue;
     }
     cudaError_t e = cudaGetLastError();
@@ -594,21 +606,21 @@ cudaError_t launch_amax(size_t npix, int C, const __nv_bfloat16* x, int ld, floa
     const unsigned cap = unsigned(device_sms()) * 8;
     if (g > cap) g = cap;
     if (g == 0) g = 1;
-    k_amax<<<g, 256, 0, s>>>(npix, C, x, ld, out);
+    launch_behind(k_amax, dim3(g), 256, 0, s, npix, C, x, ld, out);
     return cudaGetLastError();
 }
 
 cudaError_t launch_pack_features_e4m3(size_t npx, const uint8_t* rgb, const float* depth, const uint8_t* hole,
                                       const float* top3, float z_far, float s0, uint8_t* out, cudaStream_t s)
 {
-    k_pack_features_e4m3<<<blocks(npx, 256), 256, 0, s>>>(npx, rgb, depth, hole, top3, 1.0f / z_far, 1.0f / s0, out);
+    launch_behind(k_pack_features_e4m3, dim3(blocks(npx, 256)), 256, 0, s, npx, rgb, depth, hole, top3, 1.0f / z_far, 1.0f / s0, out);
     return cudaGetLastError();
 }
 
 cudaError_t launch_maxpool2_e4m3(int B, int H, int W, int C, const uint8_t* x, int ldx, uint8_t* y, cudaStream_t s)
 {
     const size_t n = size_t(B) * (H / 2) * (W / 2) * (C / 16);
-    k_maxpool2_e4m3<<<blocks(n, 256), 256, 0, s>>>(B, H, W, C, x, ldx, y);
+    launch_behind(k_maxpool2_e4m3, dim3(blocks(n, 256)), 256, 0, s, B, H, W, C, x, ldx, y);
     return cudaGetLastError();
 }
 
@@ -616,7 +628,7 @@ cudaError_t launch_flip_weights(int Cout, int Cin, const float* w, __nv_bfloat16
                                 cudaStream_t s)
 {
     const size_t n = size_t(Cout) * 9 * Cin;
-    k_flip_weights<<<blocks(n, 256), 256, 0, s>>>(Cout, Cin, w, wbf, wt);
+    launch_behind(k_flip_weights, dim3(blocks(n, 256)), 256, 0, s, Cout, Cin, w, wbf, wt);
     return cudaGetLastError();
 }
 
@@ -624,7 +636,7 @@ cudaError_t launch_sum_splits(const float* part, int splits, size_t n, float* ou
                               size_t n1, float* out2, cudaStream_t s)
 {
     if (n == 0 || splits < 1) return cudaSuccess;
-    k_sum_splits<<<unsigned((n + 31) / 32), 256, 0, s>>>(part, splits, n, out0, n0, out1, n1, out2);
+    launch_behind(k_sum_splits, dim3(unsigned((n + 31) / 32)), 256, 0, s, part, splits, n, out0, n0, out1, n1, out2);
     return cudaGetLastError();
 }
 
@@ -637,7 +649,7 @@ cudaError_t launch_adam_multi(const AdamList& L, float lr, int t, cudaStream_t s
     unsigned g = blocks(n, 256);
     const unsigned cap = unsigned(device_sms()) * 8;
     if (g > cap) g = cap;
-    k_adam_multi<<<g, 256, 0, s>>>(L, lr, b1, b2, 1e-8f, c1, c2);
+    launch_behind(k_adam_multi, dim3(g), 256, 0, s, L, lr, b1, b2, 1e-8f, c1, c2);
     return cudaGetLastError();
 }
 

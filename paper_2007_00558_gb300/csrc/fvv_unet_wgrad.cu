@@ -109,6 +109,7 @@ k_wgrad3x3_tc(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ C
     int* skip = reinterpret_cast<int*>(tmem_slot + 1);
     uint8_t* stages = base + kWgHeader;
 
+    behind();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) *skip = *reinterpret_cast<volatile int*>(P.err);
     __syncthreads();
@@ -328,12 +329,12 @@ cudaError_t launch_wgrad3x3_tc(int B, int H, int W, int Cin, int xstride, int Co
     if (halo) {
         e = cudaFuncSetAttribute(k_wgrad3x3_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, WgLayout<true>::kSmem);
         if (e != cudaSuccess) return e;
-        k_wgrad3x3_tc<true><<<grid, kWgThreads, WgLayout<true>::kSmem, s>>>(mx, mdz, a);
+        launch_behind(k_wgrad3x3_tc<true>, grid, kWgThreads, WgLayout<true>::kSmem, s, mx, mdz, a);
     } else {
         e = cudaFuncSetAttribute(k_wgrad3x3_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  WgLayout<false>::kSmem);
         if (e != cudaSuccess) return e;
-        k_wgrad3x3_tc<false><<<grid, kWgThreads, WgLayout<false>::kSmem, s>>>(mx, mdz, a);
+        launch_behind(k_wgrad3x3_tc<false>, grid, kWgThreads, WgLayout<false>::kSmem, s, mx, mdz, a);
     }
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
