@@ -507,9 +507,9 @@ __device__ __forceinline__ unsigned long long crack_rule_at(Get get, unsigned lo
     return kp;
 }
 
-// The rule on padded shared-memory rows (index -1 and Wv hold EMPTY), with up
-// the row above the pixel's.  It works on the high words alone, which are the
-// depths' bits: positive depths order like their bits, and EMPTY's high word is
+// The rule at mid, all of whose neighbours are in memory (padded rows whose
+// index -1 and Wv hold EMPTY, or a pixel off the image's border).  It works on
+// the high words alone, which are the depths' bits: positive depths order like their bits, and EMPTY's high word is
 // the largest and, as a float, a NaN, which fails every comparison it should.
 // A present pixel no deeper than (1+tau) times its nearest present neighbour
 // keeps its key without the pair walk: every consistent pair's far depth is at
@@ -519,9 +519,8 @@ __device__ __forceinline__ unsigned long long crack_rule_at(Get get, unsigned lo
 // chosen one's keys are loaded: empty pixels, which a magnified view is full
 // of, diverged at each pair before (1298x697 from
 // nine cameras 61 us then, 53 us now; 1907x1003 from five 158 and 139 us).
-__device__ __forceinline__ unsigned long long crack_rule_rows(const unsigned long long* up, int pitch, int x, float f1)
+__device__ __forceinline__ unsigned long long crack_rule_ptr(const unsigned long long* mid, int pitch, float f1)
 {
-    const unsigned long long* mid = up + pitch + x;
     const unsigned long long kp = *mid;
     const int off[4] = {1, pitch, pitch + 1, pitch - 1};             // the pairs are mid[-off], mid[off]
     auto hi = [&](int o) { return reinterpret_cast<const uint32_t*>(mid + o)[1]; };
@@ -547,21 +546,32 @@ __device__ __forceinline__ unsigned long long crack_rule_rows(const unsigned lon
 }
 
 // Layered form: the BG layer's crack filter as its own pass, read straight
-// from the z-buffer (L1/L2), so the resolve stages one key ring only.
-__global__ void __launch_bounds__(256) k_crack_bg(const ViewDesc* __restrict__ views)
+// from the z-buffer (L1/L2), so the resolve stages one key ring only.  A CTA
+// takes 64 x 4 pixels, so that its rows are read from L2 one and a half times
+// and not three (eight 1280x720 views: 64 us with
+// 256 x 1 pixels and a branch at each pair, 35 us so).
+constexpr int kBgW = 64, kBgH = 4;
+__global__ void __launch_bounds__(kBgW * kBgH) k_crack_bg(const ViewDesc* __restrict__ views)
 {
     const ViewDesc* V = views + blockIdx.z;
     const int Wv = V->Wv, Hv = V->Hv;
-    const int x = blockIdx.x * 256 + threadIdx.x, y = blockIdx.y;
+    const int x = blockIdx.x * kBgW + threadIdx.x, y = blockIdx.y * kBgH + threadIdx.y;
+    behind();
     if (x >= Wv || y >= Hv)
         return;
-    const unsigned long long* kb = V->keys_bg;
+    const unsigned long long* kb = V->keys_bg + size_t(y) * Wv + x;
     const float f1 = __fadd_rn(1.0f, V->tau_crack);
-    auto get = [&](int dy, int dx) {
-        const int yy = y + dy, xx = x + dx;
-        return (yy < 0 || yy >= Hv || xx < 0 || xx >= Wv) ? kKeyEmpty : __ldg(kb + size_t(yy) * Wv + xx);
-    };
-    V->keys_bgf[size_t(y) * Wv + x] = crack_rule_at(get, __ldg(kb + size_t(y) * Wv + x), f1);
+    unsigned long long k;
+    if (x > 0 && x < Wv - 1 && y > 0 && y < Hv - 1) {
+        k = crack_rule_ptr(kb, Wv, f1);
+    } else {
+        auto get = [&](int dy, int dx) {
+            const int yy = y + dy, xx = x + dx;
+            return (yy < 0 || yy >= Hv || xx < 0 || xx >= Wv) ? kKeyEmpty : kb[ptrdiff_t(dy) * Wv + dx];
+        };
+        k = crack_rule_at(get, *kb, f1);
+    }
+    V->keys_bgf[size_t(y) * Wv + x] = k;
 }
 
 __device__ __forceinline__ void cp_async8(void* smem_dst, const void* gsrc)
@@ -635,11 +645,18 @@ template <bool kCoh>
 __device__ __forceinline__ void gather(bool ok, const uint16_t* d, const uint32_t* c, uint32_t& dk, uint32_t& ck)
 {
     if constexpr (kCoh) {
-        dk = ck = 0u;
-        if (ok) {
-            dk = *d;
-            ck = *c;
-        }
+        asm volatile("{\n"
+                     ".reg .pred p;\n"
+                     ".reg .u16 t;\n"
+                     "setp.ne.u32 p, %4, 0;\n"
+                     "mov.u16 t, 0;\n"
+                     "mov.u32 %1, 0;\n"
+                     "@p ld.global.u16 t, [%2];\n"
+                     "@p ld.global.u32 %1, [%3];\n"
+                     "cvt.u32.u16 %0, t;\n"
+                     "}"
+                     : "=&r"(dk), "=&r"(ck)
+                     : "l"(d), "l"(c), "r"(uint32_t(ok)));
     } else {
         asm("{\n"
             ".reg .pred p;\n"
@@ -845,7 +862,7 @@ __device__ __forceinline__ void resolve_cta(const ViewDesc* __restrict__ views, 
             const int x = xb + 32 * i;
             const bool in = x < Wv;
             unsigned long long kk = kKeyEmpty;
-            if (in) kk = crack ? crack_rule_rows(up, KP, x, f1) : up[KP + x];
+            if (in) kk = crack ? crack_rule_ptr(up + KP + x, KP, f1) : up[KP + x];
             // layered: the FG layer is stacked over the BG layer, so the BG
             // layer is resolved only where the filtered FG layer is empty
             bg_layer[i] = false;
@@ -1146,7 +1163,7 @@ __device__ __forceinline__ void resolve_cta(const ViewDesc* __restrict__ views, 
                 auto depth_at = [&](int xx) {
                     if (keep) return s_dep[r * Wv + xx];
                     const unsigned long long* up = s_keys + r * KP + 2;
-                    unsigned long long kk = crack ? crack_rule_rows(up, KP, xx, f1) : up[KP + xx];
+                    unsigned long long kk = crack ? crack_rule_ptr(up + KP + xx, KP, f1) : up[KP + xx];
                     if (kLayered && kk == kKeyEmpty) kk = V->keys_bgf[rowbase + xx];
                     return key_z(kk);
                 };
@@ -1247,7 +1264,10 @@ __device__ bool persist_barrier(PersistSync* sync, unsigned int& gen, uint64_t l
 
 }  // namespace
 
-__global__ void __launch_bounds__(kResolveThreads, kResolveOcc)
+// Two CTAs of 112 registers an SM leave the 8192 that persist_grid keeps free
+// for uploads.  16 viewers of up to 1920x1080, saturated: 15,480 views/s; 10,500
+// with 80 registers, which spill, and single-row bands.
+__global__ void __maxnreg__(112)
 k_serve_persistent(PersistQueue* q, PersistSync* sync, uint32_t first, uint64_t idle_ns, uint64_t wait_ns)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -1439,10 +1459,9 @@ cudaError_t launch_warp_splat(const ViewDesc* views, int n_views, int max_chunks
 cudaError_t launch_crack_bg(const ViewDesc* views, int n_views, int max_h, int max_w, cudaStream_t stream)
 {
     if (n_views <= 0 || max_h <= 0 || max_w <= 0) return cudaSuccess;
-    dim3 grid(static_cast<unsigned>((max_w + 255) / 256), static_cast<unsigned>(max_h),
+    dim3 grid(static_cast<unsigned>((max_w + kBgW - 1) / kBgW), static_cast<unsigned>((max_h + kBgH - 1) / kBgH),
               static_cast<unsigned>(n_views));
-    k_crack_bg<<<grid, 256, 0, stream>>>(views);
-    return cudaGetLastError();
+    return launch_behind(k_crack_bg, grid, dim3(kBgW, kBgH), 0, stream, views);
 }
 
 cudaError_t launch_resolve(const ViewDesc* views, int n_views, int max_h, int max_w, int n_cams, size_t points,
@@ -1472,12 +1491,22 @@ cudaError_t launch_resolve(const ViewDesc* views, int n_views, int max_h, int ma
     return top3 ? go(k_resolve<true, false, false>) : go(k_resolve<false, false, false>);
 }
 
+// The persistent kernel's shared memory: two-row bands of the widest view where
+// two CTAs of that fit an SM, else single rows.
+namespace {
+size_t persist_smem(int max_w, int n_cams)
+{
+    const size_t two = resolve_layout(max_w, n_cams, 2, true).total;
+    return two <= 100 * 1024 ? two : resolve_layout(max_w, n_cams, 1, true).total;
+}
+}  // namespace
+
 void persist_batch_shape(int n_views, int max_h, int max_w, int n_cams, int kernel_max_w, int max_chunks, int ctas,
                          int* band, int* splat_bx)
 {
     // bands within the shared memory that the running kernel was launched
     // with; the splat's segments spread over about one virtual CTA per real one
-    *band = resolve_band(max_w, max_h, n_views, n_cams, true, ctas, resolve_layout(kernel_max_w, n_cams, 1, true).total);
+    *band = resolve_band(max_w, max_h, n_views, n_cams, true, ctas, persist_smem(kernel_max_w, n_cams));
     constexpr int kWarps = kResolveThreads / 32;
     const int need = (max_chunks + kWarps - 1) / kWarps;
     const int want = (ctas + n_views - 1) / n_views;
@@ -1486,7 +1515,7 @@ void persist_batch_shape(int n_views, int max_h, int max_w, int n_cams, int kern
 
 int persist_grid(int max_w, int n_cams)
 {
-    const size_t smem = resolve_layout(max_w, n_cams, 1, true).total;
+    const size_t smem = persist_smem(max_w, n_cams);
     int per_sm = 0;
     if (cudaFuncSetAttribute(k_serve_persistent, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) !=
             cudaSuccess ||
@@ -1515,7 +1544,7 @@ int persist_grid(int max_w, int n_cams)
 cudaError_t launch_serve_persistent(PersistQueue* q_dev, PersistSync* sync, uint32_t first, int max_w, int n_cams,
                                     uint64_t idle_ns, uint64_t wait_ns, cudaStream_t stream, int* ctas)
 {
-    const size_t smem = resolve_layout(max_w, n_cams, 1, true).total;
+    const size_t smem = persist_smem(max_w, n_cams);
     const int grid = persist_grid(max_w, n_cams);
     if (grid < 1) return cudaErrorInvalidValue;
     *ctas = grid;
