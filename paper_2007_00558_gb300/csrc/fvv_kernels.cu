@@ -81,6 +81,12 @@ constexpr int kResolveOcc = 3;                // likewise, resolve
 // code is long (eight 1080p views of three cameras 638 us with one, 719 with
 // two), but not with layers (eight 1280x720 views of five 495 and 485 us).
 constexpr int kGroup = 2;
+// The wide form: four cameras at a time in up to 128 registers, two CTAs per SM,
+// where a launch has no more CTAs than that and a gather's latency is all that
+// counts (248x158 from eight 1074x810 cameras 41.0 us for 42.9, 296x220 from
+// ten 25.4 for 26.5).  With up to four CTAs per SM it loses (one 1280x720 view
+// 84 us for 77).
+constexpr int kWideGroup = 4, kWideCtas = 2;
 constexpr int kPairs = 1;                     // pixel pairs per lane: a warp's block is 64 kPairs pixels
 constexpr int kBlock = 64 * kPairs;
 constexpr int kResolveMaxBand = 4;            // output rows per resolve CTA
@@ -712,7 +718,7 @@ __device__ __forceinline__ float pixel_weight(float cx, float cy, float cz, floa
 // weighted by the angle at its surface point) instead of the view's
 // per-camera weights.
 // ---------------------------------------------------------------------------
-template <bool kTop3, bool kLayered, bool kPixW, bool kCoh>
+template <bool kTop3, bool kLayered, bool kPixW, bool kCoh, bool kWide = false>
 __device__ __forceinline__ void resolve_cta(const ViewDesc* __restrict__ views, const FrameRef* __restrict__ frames,
                                             int band, bool keep, int bx, int by, unsigned char* smem)
 {
@@ -1091,9 +1097,11 @@ __device__ __forceinline__ void resolve_cta(const ViewDesc* __restrict__ views, 
             }
         };
         if (na > 1) {
-            constexpr int kG = kPixW && !kLayered ? 1 : kGroup;
+            constexpr int kG = kWide ? kWideGroup : kPixW && !kLayered ? 1 : kGroup;
             int a = 0;
             for (; na - a >= kG; a += kG) group(std::integral_constant<int, kG>{}, a);
+            if constexpr (kG > 2)
+                for (; na - a >= 2; a += 2) group(std::integral_constant<int, 2>{}, a);
             if (kG > 1 && a < na) group(std::integral_constant<int, 1>{}, a);
         }
 
@@ -1203,12 +1211,12 @@ __device__ __forceinline__ void resolve_cta(const ViewDesc* __restrict__ views, 
     }
 }
 
-template <bool kTop3, bool kLayered, bool kPixW>
-__global__ void __launch_bounds__(kResolveThreads, kResolveOcc)
+template <bool kTop3, bool kLayered, bool kPixW, bool kWide>
+__global__ void __launch_bounds__(kResolveThreads, kWide ? 2 : kResolveOcc)
 k_resolve(const ViewDesc* __restrict__ views, const FrameRef* __restrict__ frames, int band, int keep)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    resolve_cta<kTop3, kLayered, kPixW, false>(views, frames, band, keep != 0, int(blockIdx.x), int(blockIdx.y), smem);
+    resolve_cta<kTop3, kLayered, kPixW, false, kWide>(views, frames, band, keep != 0, int(blockIdx.x), int(blockIdx.y), smem);
 }
 
 // ---------------------------------------------------------------------------
@@ -1402,7 +1410,10 @@ namespace {
 // SM) and not for a batch.  Estimated rows of work on the busiest SM, plus the
 // start-up of each of its CTAs as kBandStart rows (717x491, eight views of 13
 // cameras: 134 us with the two rows that 0.25 gives, 141 with the four of 0.35).
-int resolve_band(int w, int h, int n_views, int n_cams, bool keep, int sms, size_t smem_cap)
+// resident: CTAs that an SM runs at once; fewer than that take as long, since a
+// lone CTA waits for its gathers (949x490 from ten 1859x1434 cameras: 131 us
+// with single rows, 208 with the four that the work alone would suggest).
+int resolve_band(int w, int h, int n_views, int n_cams, bool keep, int sms, int resident, size_t smem_cap)
 {
     int best = 1;
     double cost = 0.0;
@@ -1412,7 +1423,7 @@ int resolve_band(int w, int h, int n_views, int n_cams, bool keep, int sms, size
         const int blocks = b * ((w + kBlock - 1) / kBlock), rounds = (blocks + NW - 1) / NW;
         const double per_row = double(rounds) * NW / blocks;          // 1 when the warps fill evenly
         const long long ctas = (long long)((h + b - 1) / b) * n_views;
-        const double c = double((ctas + sms - 1) / sms) * (b * per_row + kBandStart);
+        const double c = double(std::max<long long>((ctas + sms - 1) / sms, resident)) * (b * per_row + kBandStart);
         if (b == 1 || c < cost) {
             best = b;
             cost = c;
@@ -1474,7 +1485,7 @@ cudaError_t launch_resolve(const ViewDesc* views, int n_views, int max_h, int ma
     // view: the CTAs resident at one time cover about one view, whose frames
     // stay in L2 for its gathers.
     const bool keep = double(points) < kKeepPoints * double(max_w) * double(max_h) * n_views;
-    const int band = resolve_band(max_w, max_h, n_views, n_cams, keep, device_sms(),
+    const int band = resolve_band(max_w, max_h, n_views, n_cams, keep, device_sms(), kResolveOcc,
                                   keep ? kResolveSmemKept : kResolveSmem);
     const size_t smem = resolve_layout(max_w, n_cams, band, keep).total;
     auto go = [&](auto kernel) {
@@ -1483,12 +1494,19 @@ cudaError_t launch_resolve(const ViewDesc* views, int n_views, int max_h, int ma
         dim3 grid(static_cast<unsigned>((max_h + band - 1) / band), static_cast<unsigned>(n_views));
         return launch_behind(kernel, grid, kResolveThreads, smem, stream, views, frames, band, keep ? 1 : 0);
     };
+    const bool wide = !top3 && (long long)((max_h + band - 1) / band) * n_views <= (long long)kWideCtas * device_sms();
     if (pixel_weights) {
-        if (layered) return top3 ? go(k_resolve<true, true, true>) : go(k_resolve<false, true, true>);
-        return top3 ? go(k_resolve<true, false, true>) : go(k_resolve<false, false, true>);
+        if (layered)
+            return top3 ? go(k_resolve<true, true, true, false>)
+                        : wide ? go(k_resolve<false, true, true, true>) : go(k_resolve<false, true, true, false>);
+        return top3 ? go(k_resolve<true, false, true, false>)
+                    : wide ? go(k_resolve<false, false, true, true>) : go(k_resolve<false, false, true, false>);
     }
-    if (layered) return top3 ? go(k_resolve<true, true, false>) : go(k_resolve<false, true, false>);
-    return top3 ? go(k_resolve<true, false, false>) : go(k_resolve<false, false, false>);
+    if (layered)
+        return top3 ? go(k_resolve<true, true, false, false>)
+                    : wide ? go(k_resolve<false, true, false, true>) : go(k_resolve<false, true, false, false>);
+    return top3 ? go(k_resolve<true, false, false, false>)
+                : wide ? go(k_resolve<false, false, false, true>) : go(k_resolve<false, false, false, false>);
 }
 
 // The persistent kernel's shared memory: two-row bands of the widest view where
@@ -1506,7 +1524,7 @@ void persist_batch_shape(int n_views, int max_h, int max_w, int n_cams, int kern
 {
     // bands within the shared memory that the running kernel was launched
     // with; the splat's segments spread over about one virtual CTA per real one
-    *band = resolve_band(max_w, max_h, n_views, n_cams, true, ctas, persist_smem(kernel_max_w, n_cams));
+    *band = resolve_band(max_w, max_h, n_views, n_cams, true, ctas, 1, persist_smem(kernel_max_w, n_cams));
     constexpr int kWarps = kResolveThreads / 32;
     const int need = (max_chunks + kWarps - 1) / kWarps;
     const int want = (ctas + n_views - 1) / n_views;
