@@ -59,3 +59,18 @@ def test_every_quotient_by_division(oracle_mod):
     ref = oracle_mod.synthesize(cams, rgb, dep, view, np.zeros(3), **kw)
     info = assert_parity(g, ref, "tiny coefficient")
     assert info["exact_rgb_fraction"] == 1.0
+
+
+@pytest.mark.parametrize("n", [3, 4, 6, 7])
+def test_many_rows_in_flight(oracle_mod, n):
+    """Batches whose bands outnumber two per SM: the form of two cameras at a time."""
+    rng = np.random.default_rng(40 + n)
+    cams = S.scenes.rig_arc(n, 40.0, 1.5, 80, 48, 70.0)
+    rgb, dep = _frames(rng, n, 48, 80)
+    views = [S.scenes.arc_view(-9.0 + 2.0 * i, 1.45, 97, 131, 80.0) for i in range(10)]
+    for kw in (dict(), dict(pixel_weights=1)):
+        gs = gpu_run(cams, rgb, dep, views, np.zeros(3), opts=lib().fvv_default_options(**kw))
+        for i in (0, 9):
+            ref = oracle_mod.synthesize(cams, rgb, dep, views[i], np.zeros(3), **kw)
+            info = assert_parity(gs[i], ref, "%d cameras, view %d" % (n, i))
+            assert info["exact_rgb_fraction"] == 1.0
