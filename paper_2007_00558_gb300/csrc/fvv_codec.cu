@@ -109,7 +109,9 @@ __device__ __forceinline__ void decode_block(const YuvDepth& f, const uint16_t* 
     *reinterpret_cast<uint32_t*>(r1) = c | (d << 16);
 }
 
-__global__ void __launch_bounds__(512) k_yuv_decode(YuvDepth f, int bw, int bh, uint16_t* __restrict__ out,
+// (256 threads, as large as an upload's kernel may be to run beside the persistent
+// serving kernel)
+__global__ void __launch_bounds__(256) k_yuv_decode(YuvDepth f, int bw, int bh, uint16_t* __restrict__ out,
                                                     size_t opitch)
 {
     const size_t n = size_t(bw) * bh;
@@ -332,9 +334,9 @@ cudaError_t launch_yuv_decode(const YuvDepth& f, int width, int height, uint16_t
     v.lut[0] = f.lut;
     if (vec16_ok(v, width)) return launch_decode16(v, s);
     const int sms = device_sm_count();
-    const size_t want = (n + 511) / 512;
-    const unsigned grid = unsigned(want < size_t(2 * sms) ? want : size_t(2 * sms));
-    k_yuv_decode<<<grid, 512, 0, s>>>(f, bw, bh, out, out_pitch);
+    const size_t want = (n + 255) / 256;
+    const unsigned grid = unsigned(want < size_t(4 * sms) ? want : size_t(4 * sms));
+    k_yuv_decode<<<grid, 256, 0, s>>>(f, bw, bh, out, out_pitch);
     return cudaGetLastError();
 }
 

@@ -1272,10 +1272,22 @@ __device__ bool persist_barrier(PersistSync* sync, unsigned int& gen, uint64_t l
 
 }  // namespace
 
-// Two CTAs of 112 registers an SM leave the 8192 that persist_grid keeps free
-// for uploads.  16 viewers of up to 1920x1080, saturated: 15,480 views/s; 10,500
-// with 80 registers, which spill, and single-row bands.
-__global__ void __maxnreg__(112)
+// What an upload beside the persistent kernel takes of an SM: kernels of 256
+// threads of 32 registers, or, where the context filters its depth, also the
+// depth filter's 512 threads of 32 and, as its shared memory is static, at most
+// 48 KB of that.
+constexpr size_t kSmShared = 228 * 1024, kCtaReserved = 1024;   // of an SM; what each CTA takes beside its own
+__host__ __device__ constexpr int upload_regs(bool filter) { return (filter ? 512 : 256) * 32; }
+__host__ __device__ constexpr size_t upload_smem(bool filter) { return filter ? 48 * 1024 + kCtaReserved : 0; }
+
+// Two CTAs an SM, of the registers that leave an upload its own.  16 viewers of
+// up to 1920x1080, saturated, on nine 1280x720 cameras: 15,300 views/s with 112
+// registers, 13,500 with 96 and the filter's shared memory, 10,800 with 80 (they
+// spill).  With filtered ticks at 30 Hz and 478 views/s, p99 is 0.34 to 0.6 ms and
+// the slowest view 0.5 to 3.7 ms; 19.4 and 20.4 ms where the filter has to wait
+// until the kernel idles.
+template <bool kFilter>
+__global__ void __maxnreg__(kFilter ? 96 : 112)
 k_serve_persistent(PersistQueue* q, PersistSync* sync, uint32_t first, uint64_t idle_ns, uint64_t wait_ns)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -1312,6 +1324,7 @@ k_serve_persistent(PersistQueue* q, PersistSync* sync, uint32_t first, uint64_t 
                 s_b.band = src.band;
                 s_b.splat_bx = src.splat_bx;
                 s_b.pixel_weights = src.pixel_weights;
+                s_b.keep = src.keep;
             }
         }
         __syncthreads();
@@ -1327,12 +1340,13 @@ k_serve_persistent(PersistQueue* q, PersistSync* sync, uint32_t first, uint64_t 
             splat_cta<false, false, true, kResolveThreads>(B.views, B.frames, v % B.splat_bx, v / B.splat_bx, B.splat_bx);
         if (!persist_barrier(sync, gen, wait_ns)) break;
         // (c) + (d) + (e)
+        const bool keep = kFilter ? B.keep != 0 : true;
         const int nb = (B.max_h + B.band - 1) / B.band;
         for (int v = int(blockIdx.x); v < nb * B.n_views; v += int(gridDim.x)) {
             if (B.pixel_weights)
-                resolve_cta<false, false, true, true>(B.views, B.frames, B.band, true, v % nb, v / nb, smem);
+                resolve_cta<false, false, true, true>(B.views, B.frames, B.band, keep, v % nb, v / nb, smem);
             else
-                resolve_cta<false, false, false, true>(B.views, B.frames, B.band, true, v % nb, v / nb, smem);
+                resolve_cta<false, false, false, true>(B.views, B.frames, B.band, keep, v % nb, v / nb, smem);
         }
         if (!persist_barrier(sync, gen, wait_ns)) break;
         if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -1401,6 +1415,12 @@ size_t resolve_smem_bytes(int max_w, int n_cams, bool layered)
 }
 
 namespace {
+
+// See kKeepPoints.
+bool keep_depths(size_t points, int max_w, int max_h, int n_views)
+{
+    return double(points) < kKeepPoints * double(max_w) * double(max_h) * n_views;
+}
 
 // Output rows per resolve CTA, 1..kResolveMaxBand, within smem_cap bytes.  A
 // warp takes kBlock pixels at a time, so a band's blocks should fill the eight
@@ -1484,7 +1504,7 @@ cudaError_t launch_resolve(const ViewDesc* views, int n_views, int max_h, int ma
     // view of the batch bounds every CTA's shared memory.  Launched view after
     // view: the CTAs resident at one time cover about one view, whose frames
     // stay in L2 for its gathers.
-    const bool keep = double(points) < kKeepPoints * double(max_w) * double(max_h) * n_views;
+    const bool keep = keep_depths(points, max_w, max_h, n_views);
     const int band = resolve_band(max_w, max_h, n_views, n_cams, keep, device_sms(), kResolveOcc,
                                   keep ? kResolveSmemKept : kResolveSmem);
     const size_t smem = resolve_layout(max_w, n_cams, band, keep).total;
@@ -1510,64 +1530,73 @@ cudaError_t launch_resolve(const ViewDesc* views, int n_views, int max_h, int ma
 }
 
 // The persistent kernel's shared memory: two-row bands of the widest view where
-// two CTAs of that fit an SM, else single rows.
+// two CTAs of that, and an upload, fit an SM, else single rows.  Beside the
+// filter the bands may be ones without kept depths, which leave it its room up to
+// 2024 pixels (nine cameras).
 namespace {
-size_t persist_smem(int max_w, int n_cams)
+constexpr size_t kPersistStatic = 7424;                         // at least the kernel's static shared memory
+
+size_t persist_smem(int max_w, int n_cams, bool filter)
 {
-    const size_t two = resolve_layout(max_w, n_cams, 2, true).total;
-    return two <= 100 * 1024 ? two : resolve_layout(max_w, n_cams, 1, true).total;
+    const size_t cap = std::min<size_t>(100 * 1024, (kSmShared - upload_smem(filter)) / 2 - kCtaReserved - kPersistStatic);
+    const size_t two = resolve_layout(max_w, n_cams, 2, true).total, two_lean = resolve_layout(max_w, n_cams, 2, false).total;
+    if (two <= cap) return two;
+    return filter && two_lean <= cap ? two_lean : resolve_layout(max_w, n_cams, 1, true).total;
 }
+
+auto persist_kernel(bool filter) { return filter ? k_serve_persistent<true> : k_serve_persistent<false>; }
 }  // namespace
 
-void persist_batch_shape(int n_views, int max_h, int max_w, int n_cams, int kernel_max_w, int max_chunks, int ctas,
-                         int* band, int* splat_bx)
+void persist_batch_shape(int n_views, int max_h, int max_w, int n_cams, size_t points, int kernel_max_w, bool filter,
+                         int max_chunks, int ctas, PersistBatch* batch)
 {
     // bands within the shared memory that the running kernel was launched
     // with; the splat's segments spread over about one virtual CTA per real one
-    *band = resolve_band(max_w, max_h, n_views, n_cams, true, ctas, 1, persist_smem(kernel_max_w, n_cams));
+    const bool keep = filter ? keep_depths(points, max_w, max_h, n_views) : true;
+    batch->keep = keep ? 1 : 0;
+    batch->band = resolve_band(max_w, max_h, n_views, n_cams, keep, ctas, 1, persist_smem(kernel_max_w, n_cams, filter));
     constexpr int kWarps = kResolveThreads / 32;
     const int need = (max_chunks + kWarps - 1) / kWarps;
     const int want = (ctas + n_views - 1) / n_views;
-    *splat_bx = std::max(1, std::min(need, want));
+    batch->splat_bx = std::max(1, std::min(need, want));
 }
 
-int persist_grid(int max_w, int n_cams)
+int persist_grid(int max_w, int n_cams, bool filter)
 {
-    const size_t smem = persist_smem(max_w, n_cams);
+    const size_t smem = persist_smem(max_w, n_cams, filter);
+    const auto kernel = persist_kernel(filter);
+    // An SM's split between L1 and shared memory changes only while it is idle,
+    // so what the filter needs has to be shared memory when this kernel starts.
+    cudaFuncAttributes fa{};
     int per_sm = 0;
-    if (cudaFuncSetAttribute(k_serve_persistent, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) !=
-            cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_serve_persistent, kResolveThreads, smem) !=
-            cudaSuccess) {
+    if ((filter && cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                        cudaSharedmemCarveoutMaxShared) != cudaSuccess) ||
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kResolveThreads, smem) != cudaSuccess ||
+        cudaFuncGetAttributes(&fa, kernel) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
-    // other kernels (the frame uploads: 256 threads of at most 32 registers)
-    // must fit beside the persistent one instead of waiting for it to idle:
-    // when its CTAs leave fewer registers than that, one CTA per SM less
-    cudaFuncAttributes fa{};
-    int regs_sm = 65536;
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (cudaFuncGetAttributes(&fa, k_serve_persistent) != cudaSuccess ||
-        cudaDeviceGetAttribute(&regs_sm, cudaDevAttrMaxRegistersPerMultiprocessor, dev) != cudaSuccess) {
-        cudaGetLastError();
-        return (per_sm > 1 ? per_sm - 1 : 1) * device_sms();
-    }
-    const int free_regs = regs_sm - per_sm * kResolveThreads * fa.numRegs;
-    if (free_regs < 256 * 32 && per_sm > 1) --per_sm;
+    // an upload's kernels must fit beside the persistent one instead of waiting
+    // for it to idle: when its CTAs leave fewer registers or less shared memory
+    // than they take, one CTA per SM less
+    auto fits = [&](int n) {
+        return n * kResolveThreads * fa.numRegs + upload_regs(filter) <= 65536 &&
+               size_t(n) * (smem + fa.sharedSizeBytes + kCtaReserved) + upload_smem(filter) <= kSmShared;
+    };
+    while (per_sm > 1 && !fits(per_sm)) --per_sm;
     return per_sm * device_sms();
 }
 
 cudaError_t launch_serve_persistent(PersistQueue* q_dev, PersistSync* sync, uint32_t first, int max_w, int n_cams,
-                                    uint64_t idle_ns, uint64_t wait_ns, cudaStream_t stream, int* ctas)
+                                    bool filter, uint64_t idle_ns, uint64_t wait_ns, cudaStream_t stream, int* ctas)
 {
-    const size_t smem = persist_smem(max_w, n_cams);
-    const int grid = persist_grid(max_w, n_cams);
+    const size_t smem = persist_smem(max_w, n_cams, filter);
+    const int grid = persist_grid(max_w, n_cams, filter);
     if (grid < 1) return cudaErrorInvalidValue;
     *ctas = grid;
     void* args[] = {&q_dev, &sync, &first, &idle_ns, &wait_ns};
-    return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(k_serve_persistent), dim3(unsigned(grid)),
+    return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(persist_kernel(filter)), dim3(unsigned(grid)),
                                        dim3(kResolveThreads), args, smem, stream);
 }
 
