@@ -1128,15 +1128,17 @@ fvv_status fvv_set_bg_depth(fvv_ctx* c, int32_t cam, const uint16_t* depth, size
     } else {
         if (!m) FVV_TRY(dev_alloc(c, reinterpret_cast<void**>(&m), bytes));
         c->bg[cam] = m;
-        FVV_CUDA(cudaMemset(m, 0, bytes));
-        FVV_CUDA(cudaMemcpy2D(m, size_t(c->dpitch[cam]) * 2, depth, pitch, size_t(C.width) * 2, size_t(C.height),
-                              cudaMemcpyDefault));
+        FVV_CUDA(cudaMemsetAsync(m, 0, bytes, c->own));
+        FVV_CUDA(cudaMemcpy2DAsync(m, size_t(c->dpitch[cam]) * 2, depth, pitch, size_t(C.width) * 2, size_t(C.height),
+                                   cudaMemcpyDefault, c->own));
     }
     c->bg[cam] = m;
     // every slot's frame record of this camera points at the model
     const uint16_t* p = m;
     for (int s = 0; s < c->slots; ++s)
-        FVV_CUDA(cudaMemcpy(&c->frames_dev[size_t(s) * c->n_cams + cam].bg, &p, sizeof p, cudaMemcpyHostToDevice));
+        FVV_CUDA(cudaMemcpyAsync(&c->frames_dev[size_t(s) * c->n_cams + cam].bg, &p, sizeof p, cudaMemcpyHostToDevice,
+                                 c->own));
+    FVV_CUDA(cudaStreamSynchronize(c->own));
     return FVV_OK;
 }
 

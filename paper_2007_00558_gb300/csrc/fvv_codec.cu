@@ -403,8 +403,9 @@ fvv_status fvv_set_depth_codec(fvv_ctx* c, int32_t cam, const fvv_depth_codec* p
     for (int d = 0; d < 65536; ++d) enc[d] = fvv::encode_code(d, *p, c->depth_unit_m);
     // the tables may be read by work in flight on the context's stream
     FVV_CUDA(cudaStreamSynchronize(c->own));
-    FVV_CUDA(cudaMemcpy(K->dec[cam], dec.data(), dec.size() * sizeof(uint16_t), cudaMemcpyHostToDevice));
-    FVV_CUDA(cudaMemcpy(K->enc[cam], enc.data(), enc.size() * sizeof(uint16_t), cudaMemcpyHostToDevice));
+    FVV_CUDA(cudaMemcpyAsync(K->dec[cam], dec.data(), dec.size() * sizeof(uint16_t), cudaMemcpyHostToDevice, c->own));
+    FVV_CUDA(cudaMemcpyAsync(K->enc[cam], enc.data(), enc.size() * sizeof(uint16_t), cudaMemcpyHostToDevice, c->own));
+    FVV_CUDA(cudaStreamSynchronize(c->own));
     K->prm[cam] = *p;
     K->set[cam] = 1;
     return FVV_OK;

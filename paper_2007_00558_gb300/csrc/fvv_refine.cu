@@ -43,7 +43,8 @@ fvv_status device_flag(int** out)
     std::lock_guard<std::mutex> lk(g_flag_mu);
     if (!g_flags[dev]) {
         FVV_CUDA(cudaMalloc(&g_flags[dev], sizeof(int)));
-        FVV_CUDA(cudaMemset(g_flags[dev], 0, sizeof(int)));
+        FVV_CUDA(cudaMemsetAsync(g_flags[dev], 0, sizeof(int), nullptr));
+        FVV_CUDA(cudaStreamSynchronize(nullptr));         // (streams that do not wait for this one read it)
     }
     *out = g_flags[dev];
     return FVV_OK;
@@ -195,9 +196,12 @@ fvv_status refresh_weights(RefineNet& N, cudaStream_t s)
     return FVV_OK;
 }
 
+// On the stream whose kernels read it: a plain cudaMemcpy from pageable memory
+// runs on the legacy stream, which the context's own stream does not wait for,
+// and may return before the block has arrived.
 fvv_status set_flat(RefineNet& N, Buf which, const float* in, cudaStream_t s)
 {
-    FVV_CUDA(cudaMemcpy(N.flat[int(which)], in, flat_count(N) * 4, cudaMemcpyHostToDevice));
+    FVV_CUDA(cudaMemcpyAsync(N.flat[int(which)], in, flat_count(N) * 4, cudaMemcpyHostToDevice, s));
     if (which == Buf::Param) FVV_TRY(refresh_weights(N, s));
     return FVV_OK;
 }
@@ -860,7 +864,7 @@ fvv_status fvv_refine_init(fvv_ctx* c, const fvv_unet_cfg* cfg_in)
         fvv::refine_destroy(c);
         return fail(rc, msg);
     }
-    for (auto& a : N->params) FVV_CUDA(cudaMemset(a.first, 0, a.second));
+    for (auto& a : N->params) FVV_CUDA(cudaMemsetAsync(a.first, 0, a.second, c->own));
     // He-normal 3x3 weights, zero biases, a small head
     std::mt19937_64 rng(cfg.seed);
     std::normal_distribution<float> nd(0.0f, 1.0f);
