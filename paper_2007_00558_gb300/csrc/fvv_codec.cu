@@ -269,9 +269,9 @@ __device__ __forceinline__ uint32_t chroma_of(uint32_t left, uint32_t right)
 // launch set the time; launches in a row overlap (launch_behind).  Encoding
 // nine 1280x720 frames and decoding them went from 53 to 45 us; with twice the
 // pixels a thread, so half the warps, it took 61 us.
-__global__ void __launch_bounds__(128) k_yuv_encode4(const uint16_t* __restrict__ depth, size_t dpitch, int groups,
-                                                     int bh, const uint16_t* __restrict__ lut, uint8_t* __restrict__ y,
-                                                     size_t ypitch, uint8_t* __restrict__ u, uint8_t* __restrict__ v,
+__global__ void __launch_bounds__(128) k_yuv_encode4(const uint16_t* depth, size_t dpitch, int groups,
+                                                     int bh, const uint16_t* __restrict__ lut, uint8_t* y,
+                                                     size_t ypitch, uint8_t* u, uint8_t* v,
                                                      size_t uvpitch)
 {
     launch_dependents();
@@ -282,8 +282,8 @@ __global__ void __launch_bounds__(128) k_yuv_encode4(const uint16_t* __restrict_
     uint2 q[2];
 #pragma unroll
     for (int r = 0; r < 2; ++r)
-        q[r] = __ldg(reinterpret_cast<const uint2*>(reinterpret_cast<const uint8_t*>(depth) +
-                                                    size_t(2 * by + r) * dpitch + 8 * size_t(g)));
+        q[r] = *reinterpret_cast<const uint2*>(reinterpret_cast<const uint8_t*>(depth) + size_t(2 * by + r) * dpitch +
+                                               8 * size_t(g));
     uint32_t c[2][4];
 #pragma unroll
     for (int r = 0; r < 2; ++r)

@@ -155,6 +155,12 @@ void persist_batch_shape(int n_views, int max_h, int max_w, int n_cams, size_t p
 // called launch_dependents (or exited), and calls wait_primary, which returns
 // when that kernel is complete, before it touches memory.  What overlaps is
 // the launch itself: 1.5 us of the gap between two dependent kernels.
+// Such a kernel lives while the kernels before it still write.  So it reads what
+// a kernel may have written with plain loads: no __ldg and no __restrict__, which
+// let the compiler take the read-only path, where data has to stay unwritten for
+// the whole life of the kernel, or move a load above the wait.  (Tables that the
+// host wrote, and frames and parameters that were complete before the kernel in
+// front started, may take that path.)
 #ifdef __CUDACC__
 __device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_primary() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

@@ -22,8 +22,8 @@ __device__ __forceinline__ float bf(const __nv_bfloat16 v) { return __bfloat162f
 // bytes, the smallest row a tensor map takes).  The convolution's halo copy
 // reads these 16 bytes and fills the rest of its 64-byte rows with zeros
 // (channels past the tensor's extent), so no padding lives in memory.
-__device__ __forceinline__ void features(size_t p, const uint8_t* __restrict__ rgb, const float* __restrict__ depth,
-                                         const uint8_t* __restrict__ hole, const float* __restrict__ top3,
+__device__ __forceinline__ void features(size_t p, const uint8_t* rgb, const float* depth,
+                                         const uint8_t* hole, const float* top3,
                                          float inv_zfar, float f[8])
 {
     f[0] = float(rgb[3 * p + 0]) * (1.0f / 255.0f);
@@ -36,9 +36,9 @@ __device__ __forceinline__ void features(size_t p, const uint8_t* __restrict__ r
     f[7] = top3[3 * p + 2];
 }
 
-__global__ void k_pack_features(size_t npx, const uint8_t* __restrict__ rgb, const float* __restrict__ depth,
-                                const uint8_t* __restrict__ hole, const float* __restrict__ top3, float inv_zfar,
-                                __nv_bfloat16* __restrict__ out)
+__global__ void k_pack_features(size_t npx, const uint8_t* rgb, const float* depth,
+                                const uint8_t* hole, const float* top3, float inv_zfar,
+                                __nv_bfloat16* out)
 {
     behind();
     const size_t p = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -55,9 +55,9 @@ __global__ void k_pack_features(size_t npx, const uint8_t* __restrict__ rgb, con
 }
 
 // e4m3 codes of feature / s0 in bytes 0..7, zero in 8..15
-__global__ void k_pack_features_e4m3(size_t npx, const uint8_t* __restrict__ rgb, const float* __restrict__ depth,
-                                     const uint8_t* __restrict__ hole, const float* __restrict__ top3,
-                                     float inv_zfar, float inv_s0, uint8_t* __restrict__ out)
+__global__ void k_pack_features_e4m3(size_t npx, const uint8_t* rgb, const float* depth,
+                                     const uint8_t* hole, const float* top3,
+                                     float inv_zfar, float inv_s0, uint8_t* out)
 {
     behind();
     const size_t p = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -105,8 +105,8 @@ __device__ __forceinline__ void st8(__nv_bfloat16* p, const uint4 v) { *reinterp
 // ---- pooling -----------------------------------------------------------------
 // One thread per output pixel and 8 channels.  The first maximum of the 2x2
 // window, in the order (0,0), (0,1), (1,0), (1,1), wins; its position is kept.
-__global__ void k_maxpool2(int B, int H, int W, int C, const __nv_bfloat16* __restrict__ x, int ldx,
-                           __nv_bfloat16* __restrict__ y, uint8_t* __restrict__ arg)
+__global__ void k_maxpool2(int B, int H, int W, int C, const __nv_bfloat16* x, int ldx,
+                           __nv_bfloat16* y, uint8_t* arg)
 {
     behind();
     const size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -145,9 +145,9 @@ __global__ void k_maxpool2(int B, int H, int W, int C, const __nv_bfloat16* __re
 
 // dx = route(dy by arg) + add, then zero where mask <= 0 (add, mask nullable);
 // one thread per input pixel and 8 channels
-__global__ void k_maxpool2_bwd(int B, int H, int W, int C, const __nv_bfloat16* __restrict__ dy,
-                               const uint8_t* __restrict__ arg, const __nv_bfloat16* __restrict__ add,
-                               const __nv_bfloat16* __restrict__ mask, int ldm, __nv_bfloat16* __restrict__ dx)
+__global__ void k_maxpool2_bwd(int B, int H, int W, int C, const __nv_bfloat16* dy,
+                               const uint8_t* arg, const __nv_bfloat16* add,
+                               const __nv_bfloat16* mask, int ldm, __nv_bfloat16* dx)
 {
     behind();
     const size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -183,9 +183,9 @@ __global__ void k_maxpool2_bwd(int B, int H, int W, int C, const __nv_bfloat16* 
 // ---- upsampling + concat (backward) -----------------------------------------
 // dlo = (sum over each 2x2 block of dcat[..., 0:C1]) * (lo > 0), lo read from its
 // upsampled copy up_act (full resolution, pixel stride ldu); dskip = dcat[..., C1:]
-__global__ void k_up2_concat_bwd(int B, int H, int W, int C1, int C2, const __nv_bfloat16* __restrict__ dcat,
-                                 const __nv_bfloat16* __restrict__ up_act, int ldu, __nv_bfloat16* __restrict__ dlo,
-                                 __nv_bfloat16* __restrict__ dskip)
+__global__ void k_up2_concat_bwd(int B, int H, int W, int C1, int C2, const __nv_bfloat16* dcat,
+                                 const __nv_bfloat16* up_act, int ldu, __nv_bfloat16* dlo,
+                                 __nv_bfloat16* dskip)
 {
     behind();
     const int C = C1 + C2, cv1 = C1 >> 3, cv2 = C2 >> 3;
@@ -228,8 +228,8 @@ __device__ __forceinline__ float e4m3_val(uint8_t b)
 }
 
 // 2x2 max pooling of e4m3 codes (one scale in and out); the first maximum wins
-__global__ void k_maxpool2_e4m3(int B, int H, int W, int C, const uint8_t* __restrict__ x, int ldx,
-                                uint8_t* __restrict__ y)
+__global__ void k_maxpool2_e4m3(int B, int H, int W, int C, const uint8_t* x, int ldx,
+                                uint8_t* y)
 {
     behind();
     const size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -294,9 +294,9 @@ __device__ __forceinline__ void load_d1(const uint8_t* d1, size_t p, float a[C1]
 // s = rgb / 255 + (W d1 + b); out = round(255 clamp(s, 0, 1)).  T = bf16 or
 // e4m3 codes (then scaled by s_d1).
 template <int C1, typename T>
-__global__ void k_head_fwd(size_t npx, const T* __restrict__ d1, float s_d1, const float* __restrict__ wout,
-                           const float* __restrict__ bout, const uint8_t* __restrict__ rgb, float* __restrict__ s,
-                           uint8_t* __restrict__ out, int W, size_t out_pitch, float* __restrict__ out_f32)
+__global__ void k_head_fwd(size_t npx, const T* d1, float s_d1, const float* wout,
+                           const float* bout, const uint8_t* rgb, float* s,
+                           uint8_t* out, int W, size_t out_pitch, float* out_f32)
 {
     behind();
     __shared__ float sw[3 * C1 + 3];
@@ -332,10 +332,10 @@ __global__ void k_head_fwd(size_t npx, const T* __restrict__ d1, float s_d1, con
 // owns output channels k and k + 32 of d1) and writes its partial sums to
 // part[g][3 C1 + 4] (dW, db, loss); launch_sum_splits adds them in warp order.
 template <int C1>
-__global__ void __launch_bounds__(128) k_head_bwd(size_t npx, const __nv_bfloat16* __restrict__ d1,
-                                                  const float* __restrict__ wout, const float* __restrict__ s,
-                                                  const uint8_t* __restrict__ target, float inv_count, size_t ppw,
-                                                  float* __restrict__ part, __nv_bfloat16* __restrict__ dd1)
+__global__ void __launch_bounds__(128) k_head_bwd(size_t npx, const __nv_bfloat16* d1,
+                                                  const float* wout, const float* s,
+                                                  const uint8_t* target, float inv_count, size_t ppw,
+                                                  float* part, __nv_bfloat16* dd1)
 {
     behind();
     constexpr int KPL = (C1 + 31) / 32;                 // d1 channels per lane
@@ -414,7 +414,7 @@ __global__ void __launch_bounds__(128) k_head_bwd(size_t npx, const __nv_bfloat1
 // order for 32 consecutive elements, then the eight warp sums are added in
 // warp order.  Element i goes to out0[i] (i < n0), out1[i - n0] (i < n0 + n1)
 // or out2[i - n0 - n1]; a NULL output is skipped.
-__global__ void __launch_bounds__(256) k_sum_splits(const float* __restrict__ part, int splits, size_t n,
+__global__ void __launch_bounds__(256) k_sum_splits(const float* part, int splits, size_t n,
                                                     float* out0, size_t n0, float* out1, size_t n1, float* out2)
 {
     behind();
@@ -441,8 +441,8 @@ __global__ void __launch_bounds__(256) k_sum_splits(const float* __restrict__ pa
 
 // wt[ci][ky][kx][co] = w[co][2-ky][2-kx][ci] (bf16), the weights of the
 // transposed convolution that gives the input gradient.
-__global__ void k_flip_weights(int Cout, int Cin, const float* __restrict__ w, __nv_bfloat16* __restrict__ wbf,
-                               __nv_bfloat16* __restrict__ wt)
+__global__ void k_flip_weights(int Cout, int Cin, const float* w, __nv_bfloat16* wbf,
+                               __nv_bfloat16* wt)
 {
     behind();
     const size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -492,7 +492,7 @@ __global__ void k_adam_multi(AdamList L, float lr, float b1, float b2, float eps
 
 // out = max(out, max |x|) over npix pixels of C channels at pixel stride ld
 // (out >= 0 on entry; non-negative floats order like their bits)
-__global__ void k_amax(size_t npix, int C, const __nv_bfloat16* __restrict__ x, int ld, float* __restrict__ out)
+__global__ void k_amax(size_t npix, int C, const __nv_bfloat16* x, int ld, float* out)
 {
     behind();
     const int cv = C >> 3;
