@@ -99,12 +99,11 @@ inline float settle_eps(int dim, float m0, float m1, float m2, float m3, float W
 constexpr uint32_t kZNormLoBits = 0x35800000u, kZNormHiBits = 0x5D800000u;
 constexpr float kZNormHi = 1.152921504606847e18f;
 
-// That tolerance for both directions between a W x H camera and a Wv x Hv view.
+// That tolerance for back-projections from a Wv x Hv view into a W x H camera,
+// the only ones that round without dividing (the splat divides).
 inline float map_eps(const CamGeom& G, int W, int H, int Wv, int Hv, float z_min)
 {
-    const float a = settle_eps(Wv > Hv ? Wv : Hv, G.M[8], G.M[9], G.M[10], G.M[11], float(W), float(H), 65536.0f, z_min);
-    const float b = settle_eps(W > H ? W : H, G.N[8], G.N[9], G.N[10], G.N[11], float(Wv), float(Hv), kZNormHi, z_min);
-    return a > b ? a : b;
+    return settle_eps(W > H ? W : H, G.N[8], G.N[9], G.N[10], G.N[11], float(Wv), float(Hv), kZNormHi, z_min);
 }
 
 // Persistent serving kernel (fvv_kernels.cu): one cooperative launch that

@@ -232,8 +232,8 @@ __device__ __forceinline__ float u23_to_float(uint32_t d)
 // test 0 <= t <= max as one unsigned compare per axis.  The float -> int
 // floor saturates, so +-inf and out-of-range values fail the test as in the
 // FP32 form; Z > z_min >= 0 (validated on the host) and a finite X, Y rule
-// out NaN.  This is the defining form; the kernels run it only for the few
-// points that the division-free form below does not settle.
+// out NaN.  This is the defining form: the splat runs it for every point, the
+// resolve only for the few that the division-free form below does not settle.
 __device__ __forceinline__ uint2 target_pixel_div(float X, float Y, float Z)
 {
     return make_uint2(static_cast<uint32_t>(__float2int_rd(__fadd_rn(__fdiv_rn(X, Z), 0.5f))),
@@ -321,8 +321,9 @@ __device__ __forceinline__ void round_quotient2(f32x2 X, f32x2 Z, f32x2 r, f32x2
 __device__ __forceinline__ bool target_pixel(float X, float Y, float Z, uint32_t maxu, uint32_t maxv,
                                              uint32_t& ui, uint32_t& vi)
 {
-    ui = static_cast<uint32_t>(__float2int_rd(__fadd_rn(__fdiv_rn(X, Z), 0.5f)));
-    vi = static_cast<uint32_t>(__float2int_rd(__fadd_rn(__fdiv_rn(Y, Z), 0.5f)));
+    const uint2 t = target_pixel_div(X, Y, Z);
+    ui = t.x;
+    vi = t.y;
     return ui <= maxu && vi <= maxv;
 }
 
