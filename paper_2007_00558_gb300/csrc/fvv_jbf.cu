@@ -57,8 +57,9 @@ __device__ __forceinline__ float code_to_float(uint32_t d)   // exact for d < 2^
 // wider tiles, which stage less halo per pixel, 65 us without the branch and
 // 61 us with the staging's loads in flight.  Three CTAs per SM (40 registers)
 // take 67 us.  Tiles are 128 x 16 pixels for 512 threads up to radius 3 (47 KB
-// of shared memory, four CTAs per SM); above that the arrays would pass the 48
-// KB of static shared memory, and a tile is 64 x 16.
+// of shared memory, four CTAs per SM of 32 registers a thread, which spills 52 to
+// 56 bytes); above that the arrays would pass the 48 KB of static
+// shared memory, and a tile is 64 x 16 (nothing spilled).
 constexpr int kTileH = 16;
 constexpr int kDM = 8, kCM = 32;          // left margins of the staged rows: pixels, colour bytes
 template <int R>

@@ -85,7 +85,9 @@ constexpr int kGroup = 2;
 // where a launch has no more CTAs than that and a gather's latency is all that
 // counts (248x158 from eight 1074x810 cameras 41.0 us for 42.9, 296x220 from
 // ten 25.4 for 26.5).  With up to four CTAs per SM it loses (one 1280x720 view
-// 84 us for 77).
+// 84 us for 77).  Never with the top-3 output: its lists of a pixel's largest
+// weights overfill the general form's registers as it is (24 to 44 bytes spilled;
+// four 1280x720 views of nine cameras with it 267 us, 291 with a pixel a lane).
 constexpr int kWideGroup = 4, kWideCtas = 2;
 constexpr int kPairs = 1;                     // pixel pairs per lane: a warp's block is 64 kPairs pixels
 constexpr int kBlock = 64 * kPairs;
@@ -996,7 +998,7 @@ __device__ __forceinline__ void resolve_cta(const ViewDesc* __restrict__ views, 
                     nearest = min3_abs(min3_abs(nearest, nu.x, nv.x), nu.y, nv.y);
                 }
             }
-            if (!(nearest > eps)) {                  // about one lane in 700 (six points at 1280 pixels)
+            if (!(nearest > eps)) {                  // one lane in 1000 (two cameras, four points, 1280 pixels)
 #pragma unroll 1
                 for (int a = 0; a < N; ++a) {
 #pragma unroll 1

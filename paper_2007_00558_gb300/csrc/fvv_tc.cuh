@@ -221,20 +221,6 @@ __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64
         : "memory");
 }
 
-// D[tmem] (+)= A[smem] * B[smem]^T, e4m3 inputs, fp32 accumulators (K = 32 per instruction).
-__device__ __forceinline__ void mma_e4m3(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                         uint32_t accumulate)
-{
-    asm volatile(
-        "{\n"
-        ".reg .pred p;\n"
-        "setp.ne.b32 p, %4, 0;\n"
-        "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n"
-        "}\n" ::"r"(d_tmem),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-
 // The same, called by a whole warp with uniform operands and issued by the
 // lane whose `lead` is set (always the same one).  In warp-uniform code the
 // compiler keeps descriptors in uniform registers, where the instruction
@@ -253,6 +239,7 @@ __device__ __forceinline__ void mma_bf16_lead(uint32_t d_tmem, uint64_t adesc, u
         : "memory");
 }
 
+// e4m3 inputs (K = 32 per instruction)
 __device__ __forceinline__ void mma_e4m3_lead(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                               uint32_t accumulate, uint32_t lead)
 {

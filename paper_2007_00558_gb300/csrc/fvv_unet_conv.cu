@@ -118,8 +118,9 @@ struct ConvCfg {
     static constexpr int kHaloStage = (kHaloBytes + 1023) / 1024 * 1024;   // halo slot, 1024-aligned
     // accumulator column of output row r of a tile
     __host__ __device__ static constexpr int col(int r) { return (kStack ? kRows - 1 - r : r) * kAcc; }
-    // epilogue groups: as many as a chunk's registers leave without spills (113,
-    // 146 and 200 a thread with four, three and two)
+    // epilogue groups: as many as a chunk's registers leave with few spills (96,
+    // 128 and 168 a thread with four, three and two; 4 to 12 bytes are spilled at
+    // 48 channels in bf16 and at 64 in e4m3, nothing elsewhere)
     static constexpr int kGroups = kFold ? 2 : COUT <= 32 ? 4 : COUT <= 48 ? 3 : 2;
     static constexpr int kEpiWarps = 4 * kGroups;
     static constexpr int kThreads = 64 + 32 * kEpiWarps;
