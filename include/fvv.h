@@ -359,10 +359,11 @@ fvv_status fvv_upload_frames_yuv(fvv_ctx* ctx, const uint8_t* rgb, size_t rgb_ca
  * barriers between the steps), and publishes each batch's completion in
  * that memory, where a poller thread of the library sees it.  The kernel
  * returns after idle_us without work and is launched again for the next
- * batch.  It leaves room on every SM (registers and, where jbf_radius > 0,
- * shared memory) so that the context's frame uploads run beside it.  Views may
- * be at most max_width wide (it sizes the kernel's shared memory) and outputs
- * must be device memory.  Every wait of the kernel is
+ * batch.  It leaves room on every SM (24,576 registers and 48 KB of shared
+ * memory) so that frame uploads, the depth filter and syntheses whose launches
+ * need no more run beside it; others wait until it returns.  Views may be at
+ * most max_width wide (it sizes the kernel's shared memory) and outputs must be
+ * device memory.  Every wait of the kernel is
  * bounded; a grid barrier that runs out ends the kernel and fails its
  * batches with FVV_ERR_TIMEOUT.  An upload into a frame slot that a posted
  * batch still reads waits (up to 2 s) for that batch. */

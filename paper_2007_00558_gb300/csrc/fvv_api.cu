@@ -823,8 +823,8 @@ fvv_status fvv::run_batch(fvv_ctx* c, BatchScratch& S, int n, const fvv_view* vi
             return fail(FVV_ERR_INVALID_ARG, "persistent batches take device outputs and no aux outputs");
         post->batch = PersistBatch{vdev, c->frames_dev, S.keys, koff, n, max_h, 1, 1,
                                    c->opt.pixel_weights != 0 ? 1 : 0, 1, {0, 0}};
-        fvv::persist_batch_shape(n, max_h, max_w, c->n_cams, points, post->max_width, c->opt.jbf_radius > 0,
-                                 max_chunks, post->ctas, &post->batch);
+        fvv::persist_batch_shape(n, max_h, max_w, c->n_cams, points, post->max_width, max_chunks, post->ctas,
+                                 &post->batch);
         post->slots.clear();
         for (int si = 0; si < c->slots; ++si)
             if (used[si]) post->slots.push_back(si);

@@ -137,16 +137,15 @@ constexpr int kPersistErrBarrier = 11;  // a grid barrier ran out
 // Launch the kernel on `stream` (cooperative, every CTA resident) to take
 // batches first, first + 1, ...; it returns after idle_ns without work, on
 // q->stop, or when a grid barrier waits longer than wait_ns.  max_w, n_cams
-// size its shared memory; filter: it leaves the depth filter room, too.  *ctas:
-// the grid size.
+// size its shared memory.  *ctas: the grid size.
 cudaError_t launch_serve_persistent(PersistQueue* q_dev, PersistSync* sync, uint32_t first, int max_w, int n_cams,
-                                    bool filter, uint64_t idle_ns, uint64_t wait_ns, cudaStream_t stream, int* ctas);
+                                    uint64_t idle_ns, uint64_t wait_ns, cudaStream_t stream, int* ctas);
 // The grid of that kernel for views up to max_w wide (0: none fits).
-int persist_grid(int max_w, int n_cams, bool filter);
+int persist_grid(int max_w, int n_cams);
 // The band, whether the resolve keeps depths and the splat's CTAs per view that
 // the kernel, launched for views up to kernel_max_w wide, uses for a batch
 // (points: as launch_resolve takes them).
-void persist_batch_shape(int n_views, int max_h, int max_w, int n_cams, size_t points, int kernel_max_w, bool filter,
+void persist_batch_shape(int n_views, int max_h, int max_w, int n_cams, size_t points, int kernel_max_w,
                          int max_chunks, int ctas, PersistBatch* batch);
 
 // Programmatic dependent launch: a kernel launched with launch_behind may

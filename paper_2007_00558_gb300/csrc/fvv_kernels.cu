@@ -81,14 +81,16 @@ constexpr int kResolveOcc = 3;                // likewise, resolve
 // code is long (eight 1080p views of three cameras 638 us with one, 719 with
 // two), but not with layers (eight 1280x720 views of five 495 and 485 us).
 constexpr int kGroup = 2;
-// The wide form: four cameras at a time in up to 128 registers, two CTAs per SM,
-// where a launch has no more CTAs than that and a gather's latency is all that
-// counts (248x158 from eight 1074x810 cameras 41.0 us for 42.9, 296x220 from
-// ten 25.4 for 26.5).  With up to four CTAs per SM it loses (one 1280x720 view
-// 84 us for 77).  Never with the top-3 output: its lists of a pixel's largest
-// weights overfill the general form's registers as it is (24 to 44 bytes spilled;
-// four 1280x720 views of nine cameras with it 267 us, 291 with a pixel a lane).
-constexpr int kWideGroup = 4, kWideCtas = 2;
+// The wide form: four cameras at a time, three with per-pixel weights, in up to
+// 96 registers, which the persistent serving kernel leaves beside it.  For
+// launches of at most two CTAs per SM, where a gather's latency is all that counts
+// (248x158 from eight 1074x810 cameras 41.0 us for 42.9, 296x220 from ten 25.4 for
+// 26.5; four with per-pixel weights spill, 30.9 us for 30.0).  With up to four
+// CTAs per SM it loses (one 1280x720 view 84 us for 77).  Never with the top-3
+// output: its lists of a pixel's largest weights overfill the general form's
+// registers as it is (24 to 44 bytes spilled; four 1280x720 views of nine cameras
+// with it 267 us, 291 with a pixel a lane).
+constexpr int kWideGroup = 4, kWideCtas = 2, kWideRegs = 96;
 constexpr int kPairs = 1;                     // pixel pairs per lane: a warp's block is 64 kPairs pixels
 constexpr int kBlock = 64 * kPairs;
 constexpr int kResolveMaxBand = 4;            // output rows per resolve CTA
@@ -721,7 +723,7 @@ __device__ __forceinline__ float pixel_weight(float cx, float cy, float cz, floa
 // weighted by the angle at its surface point) instead of the view's
 // per-camera weights.
 // ---------------------------------------------------------------------------
-template <bool kTop3, bool kLayered, bool kPixW, bool kCoh, bool kWide = false>
+template <bool kTop3, bool kLayered, bool kPixW, bool kCoh, int NT, bool kWide = false>
 __device__ __forceinline__ void resolve_cta(const ViewDesc* __restrict__ views, const FrameRef* __restrict__ frames,
                                             int band, bool keep, int bx, int by, unsigned char* smem)
 {
@@ -732,7 +734,7 @@ __device__ __forceinline__ void resolve_cta(const ViewDesc* __restrict__ views, 
     if (y0 >= Hv)
         return;                                    // uniform over the CTA
     const int rows = min(band, Hv - y0);
-    constexpr int NT = kResolveThreads, NW = NT / 32;
+    constexpr int NW = NT / 32;
     const int tid = threadIdx.x, lane = tid & 31;
     const int wid = __shfl_sync(0xffffffffu, tid >> 5, 0);            // uniform to the compiler, too
     const int nc = V->n_cams, na = V->n_active;
@@ -1100,7 +1102,7 @@ __device__ __forceinline__ void resolve_cta(const ViewDesc* __restrict__ views, 
             }
         };
         if (na > 1) {
-            constexpr int kG = kWide ? kWideGroup : kPixW && !kLayered ? 1 : kGroup;
+            constexpr int kG = kWide ? kWideGroup - (kPixW ? 1 : 0) : kPixW && !kLayered ? 1 : kGroup;
             int a = 0;
             for (; na - a >= kG; a += kG) group(std::integral_constant<int, kG>{}, a);
             if constexpr (kG > 2)
@@ -1214,12 +1216,22 @@ __device__ __forceinline__ void resolve_cta(const ViewDesc* __restrict__ views, 
     }
 }
 
-template <bool kTop3, bool kLayered, bool kPixW, bool kWide>
-__global__ void __launch_bounds__(kResolveThreads, kWide ? 2 : kResolveOcc)
+template <bool kTop3, bool kLayered, bool kPixW>
+__global__ void __launch_bounds__(kResolveThreads, kResolveOcc)
 k_resolve(const ViewDesc* __restrict__ views, const FrameRef* __restrict__ frames, int band, int keep)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    resolve_cta<kTop3, kLayered, kPixW, false, kWide>(views, frames, band, keep != 0, int(blockIdx.x), int(blockIdx.y), smem);
+    resolve_cta<kTop3, kLayered, kPixW, false, kResolveThreads>(views, frames, band, keep != 0, int(blockIdx.x),
+                                                                int(blockIdx.y), smem);
+}
+
+template <bool kLayered, bool kPixW>
+__global__ void __maxnreg__(kWideRegs)
+k_resolve_wide(const ViewDesc* __restrict__ views, const FrameRef* __restrict__ frames, int band, int keep)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    resolve_cta<false, kLayered, kPixW, false, kResolveThreads, true>(views, frames, band, keep != 0, int(blockIdx.x),
+                                                                      int(blockIdx.y), smem);
 }
 
 // ---------------------------------------------------------------------------
@@ -1275,22 +1287,23 @@ __device__ bool persist_barrier(PersistSync* sync, unsigned int& gen, uint64_t l
 
 }  // namespace
 
-// What an upload beside the persistent kernel takes of an SM: kernels of 256
-// threads of 32 registers, or, where the context filters its depth, also the
-// depth filter's 512 threads of 32 and, as its shared memory is static, at most
-// 48 KB of that.
+// What the persistent kernel leaves of an SM for kernels beside it, which would
+// otherwise wait until it returns: registers for a resolve in its wide form (256
+// threads of 96; the depth filter takes 512 of 32) and shared memory for the
+// filter, which as it is static has at most 48 KB.
+constexpr int kBesideRegs = kResolveThreads * kWideRegs;
 constexpr size_t kSmShared = 228 * 1024, kCtaReserved = 1024;   // of an SM; what each CTA takes beside its own
-__host__ __device__ constexpr int upload_regs(bool filter) { return (filter ? 512 : 256) * 32; }
-__host__ __device__ constexpr size_t upload_smem(bool filter) { return filter ? 48 * 1024 + kCtaReserved : 0; }
+constexpr size_t kBesideSmem = 48 * 1024 + kCtaReserved;
 
-// Two CTAs an SM, of the registers that leave an upload its own.  16 viewers of
-// up to 1920x1080, saturated, on nine 1280x720 cameras: 15,300 views/s with 112
-// registers, 13,500 with 96 and the filter's shared memory, 10,800 with 80 (they
-// spill).  With filtered ticks at 30 Hz and 478 views/s, p99 is 0.34 to 0.6 ms and
-// the slowest view 0.5 to 3.7 ms; 19.4 and 20.4 ms where the filter has to wait
-// until the kernel idles.
-template <bool kFilter>
-__global__ void __maxnreg__(kFilter ? 96 : 112)
+// Two CTAs an SM.  What is left of the registers, 40,960, serves fewer threads
+// with few spills better than more with many: 16 viewers of up to 1920x1080,
+// saturated, on nine 1280x720 cameras, 12,600 views/s with 192 threads of 104
+// registers, 10,800 with 256 of 80, 11,500 with 160 of 120, 9,700 with one CTA of
+// 384.  (256 of 112 serve 15,300, but leave 8,192: a filtered tick or a synthesis
+// beside that waits until the kernel idles.  With ticks filtered at 30 Hz and 478
+// views/s, p99 is 0.3 to 1.5 ms here and 19.4 there.)
+constexpr int kPersistThreads = 192;
+__global__ void __maxnreg__(104)
 k_serve_persistent(PersistQueue* q, PersistSync* sync, uint32_t first, uint64_t idle_ns, uint64_t wait_ns)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -1340,16 +1353,15 @@ k_serve_persistent(PersistQueue* q, PersistSync* sync, uint32_t first, uint64_t 
         if (!persist_barrier(sync, gen, wait_ns)) break;
         // (a) + (b)
         for (int v = int(blockIdx.x); v < B.splat_bx * B.n_views; v += int(gridDim.x))
-            splat_cta<false, false, true, kResolveThreads>(B.views, B.frames, v % B.splat_bx, v / B.splat_bx, B.splat_bx);
+            splat_cta<false, false, true, kPersistThreads>(B.views, B.frames, v % B.splat_bx, v / B.splat_bx, B.splat_bx);
         if (!persist_barrier(sync, gen, wait_ns)) break;
         // (c) + (d) + (e)
-        const bool keep = kFilter ? B.keep != 0 : true;
         const int nb = (B.max_h + B.band - 1) / B.band;
         for (int v = int(blockIdx.x); v < nb * B.n_views; v += int(gridDim.x)) {
             if (B.pixel_weights)
-                resolve_cta<false, false, true, true>(B.views, B.frames, B.band, keep, v % nb, v / nb, smem);
+                resolve_cta<false, false, true, true, kPersistThreads>(B.views, B.frames, B.band, B.keep != 0, v % nb, v / nb, smem);
             else
-                resolve_cta<false, false, false, true>(B.views, B.frames, B.band, keep, v % nb, v / nb, smem);
+                resolve_cta<false, false, false, true, kPersistThreads>(B.views, B.frames, B.band, B.keep != 0, v % nb, v / nb, smem);
         }
         if (!persist_barrier(sync, gen, wait_ns)) break;
         if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -1436,13 +1448,13 @@ bool keep_depths(size_t points, int max_w, int max_h, int n_views)
 // resident: CTAs that an SM runs at once; fewer than that take as long, since a
 // lone CTA waits for its gathers (949x490 from ten 1859x1434 cameras: 131 us
 // with single rows, 208 with the four that the work alone would suggest).
-int resolve_band(int w, int h, int n_views, int n_cams, bool keep, int sms, int resident, size_t smem_cap)
+int resolve_band(int w, int h, int n_views, int n_cams, bool keep, int threads, int sms, int resident, size_t smem_cap)
 {
     int best = 1;
     double cost = 0.0;
     for (int b = 1; b <= kResolveMaxBand; ++b) {
         if (b > 1 && resolve_layout(w, n_cams, b, keep).total > smem_cap) break;
-        constexpr int NW = kResolveThreads / 32;
+        const int NW = threads / 32;
         const int blocks = b * ((w + kBlock - 1) / kBlock), rounds = (blocks + NW - 1) / NW;
         const double per_row = double(rounds) * NW / blocks;          // 1 when the warps fill evenly
         const long long ctas = (long long)((h + b - 1) / b) * n_views;
@@ -1508,7 +1520,7 @@ cudaError_t launch_resolve(const ViewDesc* views, int n_views, int max_h, int ma
     // view: the CTAs resident at one time cover about one view, whose frames
     // stay in L2 for its gathers.
     const bool keep = keep_depths(points, max_w, max_h, n_views);
-    const int band = resolve_band(max_w, max_h, n_views, n_cams, keep, device_sms(), kResolveOcc,
+    const int band = resolve_band(max_w, max_h, n_views, n_cams, keep, kResolveThreads, device_sms(), kResolveOcc,
                                   keep ? kResolveSmemKept : kResolveSmem);
     const size_t smem = resolve_layout(max_w, n_cams, band, keep).total;
     auto go = [&](auto kernel) {
@@ -1518,89 +1530,84 @@ cudaError_t launch_resolve(const ViewDesc* views, int n_views, int max_h, int ma
         return launch_behind(kernel, grid, kResolveThreads, smem, stream, views, frames, band, keep ? 1 : 0);
     };
     const bool wide = !top3 && (long long)((max_h + band - 1) / band) * n_views <= (long long)kWideCtas * device_sms();
-    if (pixel_weights) {
-        if (layered)
-            return top3 ? go(k_resolve<true, true, true, false>)
-                        : wide ? go(k_resolve<false, true, true, true>) : go(k_resolve<false, true, true, false>);
-        return top3 ? go(k_resolve<true, false, true, false>)
-                    : wide ? go(k_resolve<false, false, true, true>) : go(k_resolve<false, false, true, false>);
+    if (wide) {
+        if (pixel_weights) return layered ? go(k_resolve_wide<true, true>) : go(k_resolve_wide<false, true>);
+        return layered ? go(k_resolve_wide<true, false>) : go(k_resolve_wide<false, false>);
     }
-    if (layered)
-        return top3 ? go(k_resolve<true, true, false, false>)
-                    : wide ? go(k_resolve<false, true, false, true>) : go(k_resolve<false, true, false, false>);
-    return top3 ? go(k_resolve<true, false, false, false>)
-                : wide ? go(k_resolve<false, false, false, true>) : go(k_resolve<false, false, false, false>);
+    if (pixel_weights) {
+        if (layered) return top3 ? go(k_resolve<true, true, true>) : go(k_resolve<false, true, true>);
+        return top3 ? go(k_resolve<true, false, true>) : go(k_resolve<false, false, true>);
+    }
+    if (layered) return top3 ? go(k_resolve<true, true, false>) : go(k_resolve<false, true, false>);
+    return top3 ? go(k_resolve<true, false, false>) : go(k_resolve<false, false, false>);
 }
 
 // The persistent kernel's shared memory: two-row bands of the widest view where
-// two CTAs of that, and an upload, fit an SM, else single rows.  Beside the
-// filter the bands may be ones without kept depths, which leave it its room up to
-// 2024 pixels (nine cameras).
+// two CTAs of that leave kBesideSmem (with kept depths up to 1688 pixels, without
+// up to 2024, nine cameras), else single rows.
 namespace {
 constexpr size_t kPersistStatic = 7424;                         // at least the kernel's static shared memory
 
-size_t persist_smem(int max_w, int n_cams, bool filter)
+size_t persist_smem(int max_w, int n_cams)
 {
-    const size_t cap = std::min<size_t>(100 * 1024, (kSmShared - upload_smem(filter)) / 2 - kCtaReserved - kPersistStatic);
-    const size_t two = resolve_layout(max_w, n_cams, 2, true).total, two_lean = resolve_layout(max_w, n_cams, 2, false).total;
-    if (two <= cap) return two;
-    return filter && two_lean <= cap ? two_lean : resolve_layout(max_w, n_cams, 1, true).total;
+    constexpr size_t cap = (kSmShared - kBesideSmem) / 2 - kCtaReserved - kPersistStatic;
+    for (const bool keep : {true, false}) {
+        const size_t two = resolve_layout(max_w, n_cams, 2, keep).total;
+        if (two <= cap) return two;
+    }
+    return resolve_layout(max_w, n_cams, 1, true).total;
 }
-
-auto persist_kernel(bool filter) { return filter ? k_serve_persistent<true> : k_serve_persistent<false>; }
 }  // namespace
 
-void persist_batch_shape(int n_views, int max_h, int max_w, int n_cams, size_t points, int kernel_max_w, bool filter,
+void persist_batch_shape(int n_views, int max_h, int max_w, int n_cams, size_t points, int kernel_max_w,
                          int max_chunks, int ctas, PersistBatch* batch)
 {
     // bands within the shared memory that the running kernel was launched
     // with; the splat's segments spread over about one virtual CTA per real one
-    const bool keep = filter ? keep_depths(points, max_w, max_h, n_views) : true;
+    const bool keep = keep_depths(points, max_w, max_h, n_views);
     batch->keep = keep ? 1 : 0;
-    batch->band = resolve_band(max_w, max_h, n_views, n_cams, keep, ctas, 1, persist_smem(kernel_max_w, n_cams, filter));
-    constexpr int kWarps = kResolveThreads / 32;
+    batch->band = resolve_band(max_w, max_h, n_views, n_cams, keep, kPersistThreads, ctas, 1, persist_smem(kernel_max_w, n_cams));
+    constexpr int kWarps = kPersistThreads / 32;
     const int need = (max_chunks + kWarps - 1) / kWarps;
     const int want = (ctas + n_views - 1) / n_views;
     batch->splat_bx = std::max(1, std::min(need, want));
 }
 
-int persist_grid(int max_w, int n_cams, bool filter)
+int persist_grid(int max_w, int n_cams)
 {
-    const size_t smem = persist_smem(max_w, n_cams, filter);
-    const auto kernel = persist_kernel(filter);
+    const size_t smem = persist_smem(max_w, n_cams);
     // An SM's split between L1 and shared memory changes only while it is idle,
-    // so what the filter needs has to be shared memory when this kernel starts.
+    // so what kernels beside this one need has to be shared memory when it starts.
     cudaFuncAttributes fa{};
     int per_sm = 0;
-    if ((filter && cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                        cudaSharedmemCarveoutMaxShared) != cudaSuccess) ||
-        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kResolveThreads, smem) != cudaSuccess ||
-        cudaFuncGetAttributes(&fa, kernel) != cudaSuccess) {
+    if (cudaFuncSetAttribute(k_serve_persistent, cudaFuncAttributePreferredSharedMemoryCarveout,
+                             cudaSharedmemCarveoutMaxShared) != cudaSuccess ||
+        cudaFuncSetAttribute(k_serve_persistent, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) !=
+            cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_serve_persistent, kPersistThreads, smem) !=
+            cudaSuccess ||
+        cudaFuncGetAttributes(&fa, k_serve_persistent) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
-    // an upload's kernels must fit beside the persistent one instead of waiting
-    // for it to idle: when its CTAs leave fewer registers or less shared memory
-    // than they take, one CTA per SM less
-    auto fits = [&](int n) {
-        return n * kResolveThreads * fa.numRegs + upload_regs(filter) <= 65536 &&
-               size_t(n) * (smem + fa.sharedSizeBytes + kCtaReserved) + upload_smem(filter) <= kSmShared;
+    auto leaves_room = [&](int n) {
+        return n * kPersistThreads * fa.numRegs + kBesideRegs <= 65536 &&
+               size_t(n) * (smem + fa.sharedSizeBytes + kCtaReserved) + kBesideSmem <= kSmShared;
     };
-    while (per_sm > 1 && !fits(per_sm)) --per_sm;
+    while (per_sm > 1 && !leaves_room(per_sm)) --per_sm;
     return per_sm * device_sms();
 }
 
 cudaError_t launch_serve_persistent(PersistQueue* q_dev, PersistSync* sync, uint32_t first, int max_w, int n_cams,
-                                    bool filter, uint64_t idle_ns, uint64_t wait_ns, cudaStream_t stream, int* ctas)
+                                    uint64_t idle_ns, uint64_t wait_ns, cudaStream_t stream, int* ctas)
 {
-    const size_t smem = persist_smem(max_w, n_cams, filter);
-    const int grid = persist_grid(max_w, n_cams, filter);
+    const size_t smem = persist_smem(max_w, n_cams);
+    const int grid = persist_grid(max_w, n_cams);
     if (grid < 1) return cudaErrorInvalidValue;
     *ctas = grid;
     void* args[] = {&q_dev, &sync, &first, &idle_ns, &wait_ns};
-    return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(persist_kernel(filter)), dim3(unsigned(grid)),
-                                       dim3(kResolveThreads), args, smem, stream);
+    return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(k_serve_persistent), dim3(unsigned(grid)),
+                                       dim3(kPersistThreads), args, smem, stream);
 }
 
 cudaError_t launch_pack_rgba(const uint8_t* rgb, size_t rgb_pitch, uint32_t* rgba, int rpitch,

@@ -1,5 +1,5 @@
 """The resolve kernel at the edges of its work split -- 64-pixel blocks, the two
-pixels of a lane, bands of rows, camera groups of one, two and four --
+pixels of a lane, bands of rows, camera groups of one to four --
 on the tallest view, and where every back-projection is rounded by division,
 against the oracle.  Keys, holes and depth exact, colour exact."""
 import numpy as np

@@ -1,6 +1,6 @@
-"""Frame uploads beside the persistent serving kernel: the kernel is resident on
-every SM, and a tick's kernels have to run beside it instead of waiting until it
-returns, which it does only after idle_us without work."""
+"""Frame uploads and syntheses beside the persistent serving kernel: the kernel is
+resident on every SM, and their kernels have to run beside it instead of waiting
+until it returns, which it does only after idle_us without work."""
 import time
 
 import numpy as np
@@ -73,5 +73,46 @@ def test_uploads_run_beside_the_persistent_kernel(W, radius, yuv, max_width):
         assert all(torch.equal(outs[i], alone[i]) for i in range(4)) and torch.equal(outs[4], alone[3])
         assert not torch.equal(alone[0], alone[1])
         assert max(ms) < IDLE_MS / 2, ms
+    finally:
+        F.fvv_destroy(ctx)
+
+
+# narrow views take the resolve's wide form; the outputs that a refinement needs its largest one
+@pytest.mark.parametrize("W,max_width", [(160, 160), (320, 320), (640, 640), (1280, 1280), (320, 1920)])
+@pytest.mark.parametrize("aux", [0, 1])
+def test_syntheses_run_beside_the_persistent_kernel(W, max_width, aux):
+    """As above with a view that is synthesised directly, on a stream of its own."""
+    import torch
+    F = lib()
+    h, w, n = 180, 320, 3
+    rng = np.random.default_rng(W)
+    cams = S.scenes.rig_arc(n, 40.0, 1.5, w, h, 250.0)
+    rgb = rng.integers(0, 256, (n, h, w, 3)).astype(np.uint8)
+    dep = rng.integers(1300, 1700, (n, h, w)).astype(np.uint16)
+    H = W // 2
+    view, small = S.scenes.arc_view(7.0, 1.5, W, H, 0.78 * W), S.scenes.arc_view(3.0, 1.5, 160, 96, 125.0)
+    out, alone = (torch.zeros((H, W * 3), dtype=torch.uint8, device="cuda") for _ in range(2))
+    served = torch.zeros((96, 160 * 3), dtype=torch.uint8, device="cuda")
+    t3 = torch.zeros((H, W, 3), dtype=torch.float32, device="cuda")
+    s = torch.cuda.Stream()
+    ctx = F.fvv_create(F.rig(cams, np.zeros(3)), F.fvv_default_options())
+
+    def synthesise(o):
+        F.fvv_synthesize(ctx, view, o, W * 3, F.aux(top3=t3) if aux else None, s)
+        s.synchronize()
+
+    try:
+        for k in range(n):
+            F.fvv_upload_frame(ctx, k, rgb[k], w * 3, dep[k], w * 2, 0)
+        synthesise(alone)
+        F.fvv_serve_start(ctx, F.fvv_serve_default_cfg(lanes=2, max_batch=4, memory_budget=256 << 20, persistent=1,
+                                                       max_width=max_width, idle_us=int(IDLE_MS * 1000)))
+        F.fvv_serve_poll(ctx, F.fvv_serve_submit(ctx, 0, small, served, 160 * 3), 5_000_000)       # the kernel runs
+        t0 = time.perf_counter()
+        synthesise(out)
+        ms = 1e3 * (time.perf_counter() - t0)
+        F.fvv_serve_stop(ctx)
+        assert torch.equal(out, alone)
+        assert ms < IDLE_MS / 2
     finally:
         F.fvv_destroy(ctx)
