@@ -821,8 +821,7 @@ fvv_status fvv::run_batch(fvv_ctx* c, BatchScratch& S, int n, const fvv_view* vi
     if (post) {
         if (c->opt.layered || any_host || want_top3 || aux)
             return fail(FVV_ERR_INVALID_ARG, "persistent batches take device outputs and no aux outputs");
-        post->batch = PersistBatch{vdev, c->frames_dev, S.keys, koff, n, max_h, 1, 1,
-                                   c->opt.pixel_weights != 0 ? 1 : 0, 1, {0, 0}};
+        post->batch = PersistBatch{vdev, c->frames_dev, S.keys, koff, n, max_h, 1, 1, 1, {0, 0, 0}};
         fvv::persist_batch_shape(n, max_h, max_w, c->n_cams, points, post->max_width, max_chunks, post->ctas,
                                  &post->batch);
         post->slots.clear();

@@ -117,7 +117,7 @@ struct PersistBatch {
     unsigned long long* keys;          // the batch's z-buffers, cleared first
     unsigned long long n_keys;
     int32_t n_views, max_h, band, splat_bx;
-    int32_t pixel_weights, keep, pad[2];
+    int32_t keep, pad[3];
 };
 constexpr int kPersistRing = 16;
 struct PersistQueue {
@@ -137,11 +137,13 @@ constexpr int kPersistErrBarrier = 11;  // a grid barrier ran out
 // Launch the kernel on `stream` (cooperative, every CTA resident) to take
 // batches first, first + 1, ...; it returns after idle_ns without work, on
 // q->stop, or when a grid barrier waits longer than wait_ns.  max_w, n_cams
-// size its shared memory.  *ctas: the grid size.
+// size its shared memory; pixel_weights: the context's option.  *ctas: the grid
+// size.
 cudaError_t launch_serve_persistent(PersistQueue* q_dev, PersistSync* sync, uint32_t first, int max_w, int n_cams,
-                                    uint64_t idle_ns, uint64_t wait_ns, cudaStream_t stream, int* ctas);
+                                    bool pixel_weights, uint64_t idle_ns, uint64_t wait_ns, cudaStream_t stream,
+                                    int* ctas);
 // The grid of that kernel for views up to max_w wide (0: none fits).
-int persist_grid(int max_w, int n_cams);
+int persist_grid(int max_w, int n_cams, bool pixel_weights);
 // The band, whether the resolve keeps depths and the splat's CTAs per view that
 // the kernel, launched for views up to kernel_max_w wide, uses for a batch
 // (points: as launch_resolve takes them).

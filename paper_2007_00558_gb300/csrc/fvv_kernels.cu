@@ -817,7 +817,7 @@ __device__ __forceinline__ void resolve_cta(const ViewDesc* __restrict__ views, 
         const float fy = u23_to_float(uint32_t(y0 + r));
         s_row[i] = make_float4(__fmul_rn(N[1], fy), __fmul_rn(N[5], fy), __fmul_rn(N[9], fy), 0.0f);
     }
-    if (!kLayered && V->keys_next) {
+    if (!kLayered && !kCoh && V->keys_next) {
         // the next batch's z-buffer rows of this band, emptied while the key
         // rows are in flight (kept in L2 for that batch's splat); the buffer
         // starts on a 128-byte line, so even keys pair up
@@ -841,8 +841,9 @@ __device__ __forceinline__ void resolve_cta(const ViewDesc* __restrict__ views, 
     const float tau_vis = V->tau_vis, zmin = V->z_min;
     const uint32_t dlo = V->d_lo, dspan = V->d_hi - V->d_lo;
     float* __restrict__ top3 = V->out_top3;
-    float* __restrict__ odepth = V->out_depth;
-    unsigned long long* __restrict__ okeys = V->out_keys;
+    // (the persistent kernel's views have no outputs but the colour, and no next z-buffer)
+    float* __restrict__ odepth = kCoh ? nullptr : V->out_depth;
+    unsigned long long* __restrict__ okeys = kCoh ? nullptr : V->out_keys;
     const f32x2 nz = neg_zero2();
     const float eps = V->eps;
     cp_async_wait<0>();
@@ -1211,7 +1212,7 @@ __device__ __forceinline__ void resolve_cta(const ViewDesc* __restrict__ views, 
             orow[i] = uint8_t(c_rgb[x] >> (8 * (i - 3 * x)));
         }
         const size_t rowbase = size_t(y) * Wv;
-        if (V->out_hole)
+        if (!kCoh && V->out_hole)
             for (int x = tid; x < Wv; x += NT) V->out_hole[rowbase + x] = uint8_t((c_rgb[x] & kHoleBit) >> 24);
     }
 }
@@ -1289,20 +1290,24 @@ __device__ bool persist_barrier(PersistSync* sync, unsigned int& gen, uint64_t l
 
 // What the persistent kernel leaves of an SM for kernels beside it, which would
 // otherwise wait until it returns: registers for a resolve in its wide form (256
-// threads of 96; the depth filter takes 512 of 32) and shared memory for the
-// filter, which as it is static has at most 48 KB.
+// threads of 96, two warps to each quarter of the SM; the depth filter takes 512
+// of 32) and shared memory for the filter, which as it is static has at most 48 KB.
 constexpr int kBesideRegs = kResolveThreads * kWideRegs;
 constexpr size_t kSmShared = 228 * 1024, kCtaReserved = 1024;   // of an SM; what each CTA takes beside its own
 constexpr size_t kBesideSmem = 48 * 1024 + kCtaReserved;
 
-// Two CTAs an SM.  What is left of the registers, 40,960, serves fewer threads
-// with few spills better than more with many: 16 viewers of up to 1920x1080,
-// saturated, on nine 1280x720 cameras, 12,600 views/s with 192 threads of 104
-// registers, 10,800 with 256 of 80, 11,500 with 160 of 120, 9,700 with one CTA of
-// 384.  (256 of 112 serve 15,300, but leave 8,192: a filtered tick or a synthesis
-// beside that waits until the kernel idles.  With ticks filtered at 30 Hz and 478
-// views/s, p99 is 0.3 to 1.5 ms here and 19.4 there.)
+// Two CTAs an SM, three warps of each quarter.  What is left of the registers,
+// 40,960, serves fewer threads without spills better than more with them: 16
+// viewers of up to 1920x1080, saturated, on nine 1280x720 cameras, 12,950 views/s
+// with 192 threads of 104 registers, 12,750 with 256 of 80, 11,500 with 160 of
+// 120, 9,700 with one CTA of 384.  (224 of 88 serve 13,300, but put four warps on
+// some quarters, beside which the wide form does not fit.  256 of 112 serve
+// 15,300, but a filtered tick or a synthesis beside that waits until the kernel
+// idles: with ticks filtered at 30 Hz and 478 views/s, p99 is 0.3 to 1.5 ms here
+// and 19.4 there.)  The two kinds of weights are instances, as both in one kernel
+// spill (12,650).
 constexpr int kPersistThreads = 192;
+template <bool kPixW>
 __global__ void __maxnreg__(104)
 k_serve_persistent(PersistQueue* q, PersistSync* sync, uint32_t first, uint64_t idle_ns, uint64_t wait_ns)
 {
@@ -1339,7 +1344,6 @@ k_serve_persistent(PersistQueue* q, PersistSync* sync, uint32_t first, uint64_t 
                 s_b.max_h = src.max_h;
                 s_b.band = src.band;
                 s_b.splat_bx = src.splat_bx;
-                s_b.pixel_weights = src.pixel_weights;
                 s_b.keep = src.keep;
             }
         }
@@ -1357,12 +1361,8 @@ k_serve_persistent(PersistQueue* q, PersistSync* sync, uint32_t first, uint64_t 
         if (!persist_barrier(sync, gen, wait_ns)) break;
         // (c) + (d) + (e)
         const int nb = (B.max_h + B.band - 1) / B.band;
-        for (int v = int(blockIdx.x); v < nb * B.n_views; v += int(gridDim.x)) {
-            if (B.pixel_weights)
-                resolve_cta<false, false, true, true, kPersistThreads>(B.views, B.frames, B.band, B.keep != 0, v % nb, v / nb, smem);
-            else
-                resolve_cta<false, false, false, true, kPersistThreads>(B.views, B.frames, B.band, B.keep != 0, v % nb, v / nb, smem);
-        }
+        for (int v = int(blockIdx.x); v < nb * B.n_views; v += int(gridDim.x))
+            resolve_cta<false, false, kPixW, true, kPersistThreads>(B.views, B.frames, B.band, B.keep != 0, v % nb, v / nb, smem);
         if (!persist_barrier(sync, gen, wait_ns)) break;
         if (blockIdx.x == 0 && threadIdx.x == 0) {
             __threadfence_system();           // the batch's outputs before its completion
@@ -1557,6 +1557,11 @@ size_t persist_smem(int max_w, int n_cams)
     }
     return resolve_layout(max_w, n_cams, 1, true).total;
 }
+
+auto persist_kernel(bool pixel_weights)
+{
+    return pixel_weights ? k_serve_persistent<true> : k_serve_persistent<false>;
+}
 }  // namespace
 
 void persist_batch_shape(int n_views, int max_h, int max_w, int n_cams, size_t points, int kernel_max_w,
@@ -1573,25 +1578,26 @@ void persist_batch_shape(int n_views, int max_h, int max_w, int n_cams, size_t p
     batch->splat_bx = std::max(1, std::min(need, want));
 }
 
-int persist_grid(int max_w, int n_cams)
+int persist_grid(int max_w, int n_cams, bool pixel_weights)
 {
+    const auto kernel = persist_kernel(pixel_weights);
     const size_t smem = persist_smem(max_w, n_cams);
     // An SM's split between L1 and shared memory changes only while it is idle,
     // so what kernels beside this one need has to be shared memory when it starts.
     cudaFuncAttributes fa{};
     int per_sm = 0;
-    if (cudaFuncSetAttribute(k_serve_persistent, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             cudaSharedmemCarveoutMaxShared) != cudaSuccess ||
-        cudaFuncSetAttribute(k_serve_persistent, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) !=
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) !=
             cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_serve_persistent, kPersistThreads, smem) !=
-            cudaSuccess ||
-        cudaFuncGetAttributes(&fa, k_serve_persistent) != cudaSuccess) {
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kPersistThreads, smem) != cudaSuccess ||
+        cudaFuncGetAttributes(&fa, kernel) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
     auto leaves_room = [&](int n) {
-        return n * kPersistThreads * fa.numRegs + kBesideRegs <= 65536 &&
+        // registers belong to the quarters of an SM, and a CTA's warps to one each in turn
+        const int warps = n * kPersistThreads / 32, quarter = (warps + 3) / 4 * 32 * fa.numRegs;
+        return quarter + kBesideRegs / 4 <= 65536 / 4 &&
                size_t(n) * (smem + fa.sharedSizeBytes + kCtaReserved) + kBesideSmem <= kSmShared;
     };
     while (per_sm > 1 && !leaves_room(per_sm)) --per_sm;
@@ -1599,14 +1605,15 @@ int persist_grid(int max_w, int n_cams)
 }
 
 cudaError_t launch_serve_persistent(PersistQueue* q_dev, PersistSync* sync, uint32_t first, int max_w, int n_cams,
-                                    uint64_t idle_ns, uint64_t wait_ns, cudaStream_t stream, int* ctas)
+                                    bool pixel_weights, uint64_t idle_ns, uint64_t wait_ns, cudaStream_t stream,
+                                    int* ctas)
 {
     const size_t smem = persist_smem(max_w, n_cams);
-    const int grid = persist_grid(max_w, n_cams);
+    const int grid = persist_grid(max_w, n_cams, pixel_weights);
     if (grid < 1) return cudaErrorInvalidValue;
     *ctas = grid;
     void* args[] = {&q_dev, &sync, &first, &idle_ns, &wait_ns};
-    return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(k_serve_persistent), dim3(unsigned(grid)),
+    return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(persist_kernel(pixel_weights)), dim3(unsigned(grid)),
                                        dim3(kPersistThreads), args, smem, stream);
 }
 

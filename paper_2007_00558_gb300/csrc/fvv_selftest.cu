@@ -77,7 +77,7 @@ fvv_status fvv_selftest_persistent_wait(int32_t barrier, uint32_t limit_us, void
     int ctas = 0;
     const uint64_t ns = uint64_t(limit_us) * 1000ull;
     if (e == cudaSuccess)
-        e = fvv::launch_serve_persistent(qd, sync, 0, 64, 1, barrier ? 2000000000ull : ns,
+        e = fvv::launch_serve_persistent(qd, sync, 0, 64, 1, false, barrier ? 2000000000ull : ns,
                                          barrier ? ns : ns + 2000000000ull, s, &ctas);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     const int err = q->err;

@@ -152,7 +152,7 @@ fvv_status persist_launch(fvv_ctx* c, ServeState* st)
     const uint64_t idle_ns = uint64_t(st->cfg.idle_us) * 1000ull;
     const uint64_t wait_ns = std::max<uint64_t>(kPersistBarrierNs, idle_ns + 1000000000ull);
     const cudaError_t e = launch_serve_persistent(st->pq_dev, st->psync, st->pq->done, st->cfg.max_width, c->n_cams,
-                                                  idle_ns, wait_ns, st->pstream, &ctas);
+                                                  c->opt.pixel_weights != 0, idle_ns, wait_ns, st->pstream, &ctas);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return fail(FVV_ERR_CUDA, std::string("persistent serving kernel: ") + cudaGetErrorString(e));
@@ -785,7 +785,7 @@ fvv_status fvv_serve_start(fvv_ctx* c, const fvv_serve_cfg* cfg_in)
             return unwind(FVV_ERR_OUT_OF_MEMORY, fvv_last_error());
         }
         st->psync = static_cast<fvv::PersistSync*>(ps);
-        st->pctas = fvv::persist_grid(cfg.max_width, c->n_cams);
+        st->pctas = fvv::persist_grid(cfg.max_width, c->n_cams, c->opt.pixel_weights != 0);
         if (st->pctas < 1) {
             cudaFreeHost(st->pq);
             st->pq = nullptr;

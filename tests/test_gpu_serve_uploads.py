@@ -81,7 +81,8 @@ def test_uploads_run_beside_the_persistent_kernel(W, radius, yuv, max_width):
 @pytest.mark.parametrize("W,max_width", [(160, 160), (320, 320), (640, 640), (1280, 1280), (320, 1920)])
 @pytest.mark.parametrize("aux", [0, 1])
 def test_syntheses_run_beside_the_persistent_kernel(W, max_width, aux):
-    """As above with a view that is synthesised directly, on a stream of its own."""
+    """As above with a view that is synthesised directly, on a stream of its own
+    (aux: with the top-3 weights and per-pixel angular weights)."""
     import torch
     F = lib()
     h, w, n = 180, 320, 3
@@ -92,10 +93,10 @@ def test_syntheses_run_beside_the_persistent_kernel(W, max_width, aux):
     H = W // 2
     view, small = S.scenes.arc_view(7.0, 1.5, W, H, 0.78 * W), S.scenes.arc_view(3.0, 1.5, 160, 96, 125.0)
     out, alone = (torch.zeros((H, W * 3), dtype=torch.uint8, device="cuda") for _ in range(2))
-    served = torch.zeros((96, 160 * 3), dtype=torch.uint8, device="cuda")
+    served, ref = (torch.zeros((96, 160 * 3), dtype=torch.uint8, device="cuda") for _ in range(2))
     t3 = torch.zeros((H, W, 3), dtype=torch.float32, device="cuda")
     s = torch.cuda.Stream()
-    ctx = F.fvv_create(F.rig(cams, np.zeros(3)), F.fvv_default_options())
+    ctx = F.fvv_create(F.rig(cams, np.zeros(3)), F.fvv_default_options(pixel_weights=aux))
 
     def synthesise(o):
         F.fvv_synthesize(ctx, view, o, W * 3, F.aux(top3=t3) if aux else None, s)
@@ -105,6 +106,8 @@ def test_syntheses_run_beside_the_persistent_kernel(W, max_width, aux):
         for k in range(n):
             F.fvv_upload_frame(ctx, k, rgb[k], w * 3, dep[k], w * 2, 0)
         synthesise(alone)
+        F.fvv_synthesize(ctx, small, ref, 160 * 3, None, s)
+        s.synchronize()
         F.fvv_serve_start(ctx, F.fvv_serve_default_cfg(lanes=2, max_batch=4, memory_budget=256 << 20, persistent=1,
                                                        max_width=max_width, idle_us=int(IDLE_MS * 1000)))
         F.fvv_serve_poll(ctx, F.fvv_serve_submit(ctx, 0, small, served, 160 * 3), 5_000_000)       # the kernel runs
@@ -112,7 +115,7 @@ def test_syntheses_run_beside_the_persistent_kernel(W, max_width, aux):
         synthesise(out)
         ms = 1e3 * (time.perf_counter() - t0)
         F.fvv_serve_stop(ctx)
-        assert torch.equal(out, alone)
+        assert torch.equal(out, alone) and torch.equal(served, ref)
         assert ms < IDLE_MS / 2
     finally:
         F.fvv_destroy(ctx)
